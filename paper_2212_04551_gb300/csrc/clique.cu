@@ -382,11 +382,18 @@ void run_clique(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_
     if (k_lo < 1 || k_hi > GPM_CLIQUE_MAX_K || k_lo > k_hi) fail(GPM_EINVAL, "bad clique size range");
     ensure_dag(g);
     cudaStream_t s = g->stream;
+    const bool whole = !d_roots;
     if (!d_roots) {
         d_roots = ensure_root_order(g, GPM_APP_CLIQUE);
         n_roots = g->n;
         n_counter = -1;
     }
+    // Whole-graph counts branch on non-edges (clique_nonedge.cu) instead of
+    // walking the cliques.  Root lists, schedules and per-root results keep
+    // the walk below, whose units, hand-offs and bounded waits they are
+    // defined on, and so does a caller that chooses one of the walk's tails.
+    const bool nonedge = whole && !d_per_root && k_hi >= 3 && g->cfg.clique_cpl != 0 && g->cfg.clique_tail == 0 &&
+                         g->cfg.clique_compact == 0;
     if (n_counter < 0 || n_counter > n_roots) n_counter = n_roots;
     const int n_split = (int)(n_roots - n_counter);
     const int split_chunks = plan ? plan->chunks : 0;
@@ -404,6 +411,8 @@ void run_clique(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_
         GPM_CUDA(cudaMemsetAsync(d_per_root, 0, sizeof(unsigned long long) * n_roots, s));
 
     gpm_stats st{};
+    int launches = 0;
+    bool timed = false;
     if (k_hi <= 2) {
         // k = 1: one per root; k = 2: its out-degree (single sizes only)
         if (k_lo != k_hi) fail(GPM_EINVAL, "range counting needs k_lo >= 3");
@@ -412,6 +421,15 @@ void run_clique(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_
                 g->dag_outdeg.as<int32_t>(), d_roots, n_roots, k_hi, d_per_root, ctl);
             GPM_CUDA(cudaGetLastError());
         }
+    } else if (n_roots > 0 && nonedge) {
+        Grid gr;
+        GPM_CUDA(cudaEventRecord(g->ev0, s));
+        launches = launch_clique_nonedge(g, k_lo, k_hi, ctl, &gr);
+        run_clique_list(g, k_lo, k_hi, d_roots, n_roots, d_per_root, ctl, CQ_MAX_OUTDEG);
+        GPM_CUDA(cudaEventRecord(g->ev1, s));
+        timed = true;
+        st.grid_blocks = gr.blocks;
+        st.warps_per_block = gr.warps_per_block;
     } else if (n_roots > 0) {
         CliqueLaunch L = plan_clique_launch(g, k_lo, k_hi, d_roots, n_counter, n_seed, 0);
         CliqueParams& p = L.p;
@@ -425,12 +443,14 @@ void run_clique(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_
         GPM_CUDA(cudaGetLastError());
         run_clique_list(g, k_lo, k_hi, d_roots, n_roots, d_per_root, ctl, CQ_MAX_OUTDEG);
         GPM_CUDA(cudaEventRecord(g->ev1, s));
+        launches = n_split > 0 ? 3 : 2;
+        timed = true;
         st.grid_blocks = L.gr.blocks;
         st.warps_per_block = L.wpb;
     }
     GPM_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(Control), cudaMemcpyDeviceToHost, s));
     GPM_CUDA(cudaStreamSynchronize(s));
-    if (st.grid_blocks) {
+    if (timed) {
         float ms = 0.f;
         GPM_CUDA(cudaEventElapsedTime(&ms, g->ev0, g->ev1));
         st.kernel_ms = ms;
@@ -440,8 +460,8 @@ void run_clique(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_
     st.idle_polls = h.idle_polls;
     st.word_ops = h.word_ops;
     st.busy_warp_ns = h.busy_ns;
-    st.kernel_launches = st.grid_blocks ? (n_split > 0 ? 3 : 2) : (k_hi <= 2 && n_roots > 0 ? 1 : 0);
-    if (st.grid_blocks && g->max_outdeg > CQ_MAX_OUTDEG) st.kernel_launches += 2;   // the list path
+    st.kernel_launches = k_hi <= 2 && n_roots > 0 ? 1 : launches;
+    if (timed && g->max_outdeg > CQ_MAX_OUTDEG) st.kernel_launches += 2;   // the list path
     g->stats = st;
     if (h.error == DEV_ETIMEOUT) fail(GPM_ETIMEOUT, "an idle warp waited longer than max_idle_ms without progress");
     if (h.error) fail(GPM_ECUDA, "device error " + std::to_string(h.error));

@@ -91,6 +91,7 @@ struct gpm_graph {
     // root orders of the plain scheduler (built lazily)
     bool order_motif_ready = false, order_clique_ready = false;
     gpm::DevBuf order_motif, order_clique;
+    std::vector<int32_t> order_clique_starts;   // where each out-degree begins in order_clique
     bool order_id_ready = false;
     gpm::DevBuf order_id;
     // custom root order (learned scheduler or caller)
@@ -171,6 +172,7 @@ struct Grid {
 void ensure_dag(gpm_graph* g);
 const int32_t* ensure_root_order(gpm_graph* g, int app);  // plain scheduler order
 const int32_t* ensure_id_order(gpm_graph* g);             // 0, 1, ..., n-1
+long long roots_at_least(gpm_graph* g, int d);            // vertices of out-degree >= d: the first ones of the clique order
 void exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, int64_t* total,
                         cudaStream_t s, DevBuf& tmp);
 
@@ -208,6 +210,9 @@ void run_clique_dfs(gpm_graph* g, int k, uint64_t* count_out);   // the paper's 
 // by list intersection after the bitmap launch (same Control, same counters)
 void run_clique_list(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_t n_roots,
                      unsigned long long* d_per_root, Control* ctl, int bitmap_limit);
+// clique_nonedge.cu: whole-graph counts of sizes k_lo .. k_hi (k_hi >= 3) into
+// ctl, without the roots above the bitmap limit; returns the launches made
+int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* grid);
 void run_motif_monitored(gpm_graph* g, int k, double threshold, uint64_t* counts_out, MonitorStats* ms);
 
 // clique.cu / motif.cu

@@ -281,8 +281,11 @@ static int grid_for(int64_t work, int threads, int sms) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)sms * 32));
 }
 
-// vertices sorted by key descending (ties in no particular order)
-static void order_by_key_desc(gpm_graph* g, const int32_t* key, int32_t maxkey, DevBuf& out) {
+// vertices sorted by key descending (ties in no particular order); starts
+// (nullable) receives the position where each key begins: starts[j] vertices
+// have a key above maxkey - j
+static void order_by_key_desc(gpm_graph* g, const int32_t* key, int32_t maxkey, DevBuf& out,
+                              std::vector<int32_t>* starts = nullptr) {
     cudaStream_t s = g->stream;
     const int32_t n = g->n;
     out.ensure(sizeof(int32_t) * std::max(n, 1));
@@ -294,6 +297,11 @@ static void order_by_key_desc(gpm_graph* g, const int32_t* key, int32_t maxkey, 
         k_key_hist<<<grid_for(n, 256, g->num_sms), 256, 0, s>>>(key, n, maxkey, hist.as<int32_t>());
         int64_t total = 0;
         exclusive_scan_i32(hist.as<int32_t>(), cur.as<int32_t>(), maxkey + 1, &total, s, tmp);
+        if (starts) {
+            starts->resize((size_t)maxkey + 2);
+            GPM_CUDA(cudaMemcpyAsync(starts->data(), cur.ptr, sizeof(int32_t) * starts->size(), cudaMemcpyDeviceToHost,
+                                     s));
+        }
         k_key_scatter<<<grid_for(n, 256, g->num_sms), 256, 0, s>>>(key, n, maxkey, cur.as<int32_t>(),
                                                                    out.as<int32_t>());
         GPM_CUDA(cudaGetLastError());
@@ -339,7 +347,8 @@ const int32_t* ensure_root_order(gpm_graph* g, int app) {
     if (app == GPM_APP_CLIQUE) {
         ensure_dag(g);
         if (!g->order_clique_ready) {
-            order_by_key_desc(g, g->dag_outdeg.as<int32_t>(), std::max(g->max_outdeg, 0), g->order_clique);
+            order_by_key_desc(g, g->dag_outdeg.as<int32_t>(), std::max(g->max_outdeg, 0), g->order_clique,
+                              &g->order_clique_starts);
             g->order_clique_ready = true;
         }
         return g->order_clique.as<int32_t>();
@@ -349,6 +358,13 @@ const int32_t* ensure_root_order(gpm_graph* g, int app) {
         g->order_motif_ready = true;
     }
     return g->order_motif.as<int32_t>();
+}
+
+long long roots_at_least(gpm_graph* g, int d) {
+    ensure_root_order(g, GPM_APP_CLIQUE);
+    if (d <= 0) return g->n;
+    if (g->n == 0 || d > g->max_outdeg) return 0;
+    return g->order_clique_starts[(size_t)(g->max_outdeg - d + 1)];
 }
 
 __global__ void k_iota(int32_t* out, int32_t n) {
