@@ -14,6 +14,11 @@
 // the launch (batch_split); warps simply leave when the unit counter runs out
 // -- no waiting at all.
 //
+// Motifs of 3 .. 5 vertices are counted by the homomorphism kernel instead
+// (motif_hom.cu), a second launch of the same capture over all vertices: a
+// warp's sums are added to its graph's when the next vertex belongs to
+// another, and a last launch turns them into pattern counts.
+//
 // The launch (counter resets, kernel, read-back) is captured once into a CUDA
 // graph per (clique k, motif k, launch shape) and replayed on every call.  An
 // autotuner times the replay over warps per block, resident blocks per SM,
@@ -30,6 +35,7 @@
 #include "clique_dev.cuh"
 #include "common.cuh"
 #include "motif_dev.cuh"
+#include "motif_hom.cuh"
 
 namespace gpm {
 gpm_graph* create_graph(const int32_t* indptr, const int32_t* indices, int32_t n, uint32_t flags, void* stream);
@@ -50,9 +56,10 @@ struct gpm_batch {
         cudaGraphExec_t exec = nullptr;
         gpm::DevBuf units, uranges;  // this launch's unit list (baked into the graph)
         gpm::DevBuf dev_out;         // [G] clique + [G*npat] motif + Control
+        gpm::DevBuf dev_hom;         // [G][HOM_N] homomorphism sums, then the launch's ticket
         unsigned long long* host_out = nullptr;   // pinned
         size_t words = 0;
-        int blocks = 0, wpb = 0;
+        int blocks = 0, wpb = 0, launches = 0;
     };
     // (kc, km, wpb, bps, order, motif_agg_min, batch_split)
     std::map<std::tuple<int, int, int, int, int, int, int>, Captured> graphs;
@@ -298,8 +305,11 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
 
     if (kc > 0) ensure_dag(g);
     DevBuf units, uranges;
-    const long long n_units = build_units(b, kc, km, b->order_mode, split, units, uranges);
     const int npat = km > 0 ? (int)pattern_table(km).num_patterns : 0;
+    const int hom_k = km;
+    const bool hom = km > 0 && b->cfg.motif_agg_min > 0 && hom_applies(b->max_graph_n, g->max_deg, km);
+    if (hom) km = 0;      // no motif units in k_batch
+    const long long n_units = build_units(b, kc, km, b->order_mode, split, units, uranges);
 
     BatchParams p{};
     p.indptr = g->indptr.as<int32_t>();
@@ -315,28 +325,34 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     p.n_units = n_units;
     p.kc = kc;
     p.km = km;
-    p.npat = npat;
     p.lut = km > 0 ? device_lut(km) : nullptr;
     if (kc > 0 && g->max_outdeg > 1024) fail(GPM_ENOTIMPL, "batched clique counting needs out-degrees <= 1024");
     p.cq_maxd = std::max(kc > 0 ? g->max_outdeg : 1, 1);
     p.cq_wmax = (p.cq_maxd + 31) / 32;
     p.cq_words = cq_layout(p.cq_maxd, p.cq_wmax, false).total;
-    p.mark_stride = (b->max_graph_n + 15) & ~15;
-    long long off = 0;
-    const long long D = std::max(g->max_deg, 1);
-    for (int l = 0; l <= MT_MAXK; l++) {
-        p.lvl_off[l] = off;
-        if (km > 0 && l >= 1 && l <= km - 2) off += (long long)l * D + 4;
-        off = (off + 3) & ~3ll;
-    }
-    p.slab_ints = (int)std::max(off, 4ll);
-    p.agg_min = b->cfg.motif_agg_min;
-    p.agg_words = (km > 0 && p.agg_min > 0) ? mt_agg_words(km) : 0;
-    const size_t mt_bytes = ((sizeof(MtWarp) + 15) & ~size_t(15)) + sizeof(unsigned long long) * ((npat + 1) & ~1) +
-                            4 * (size_t)((p.agg_words + 3) & ~3) + p.mark_stride + 4 * (size_t)p.slab_ints;
-    p.warp_bytes = (int)((p.cq_words * 4 + mt_bytes + 15) & ~size_t(15));
-    const size_t smem = (size_t)wpb * p.warp_bytes;
+    // shared memory of a warp with motif size m in the launch (0: none)
+    auto layout = [&](int m) {
+        p.mark_stride = m > 0 ? (b->max_graph_n + 15) & ~15 : 16;
+        long long off = 0;
+        const long long D = std::max(g->max_deg, 1);
+        for (int l = 0; l <= MT_MAXK; l++) {
+            p.lvl_off[l] = off;
+            if (m > 0 && l >= 1 && l <= m - 2) off += (long long)l * D + 4;
+            off = (off + 3) & ~3ll;
+        }
+        p.slab_ints = (int)std::max(off, 4ll);
+        p.agg_min = b->cfg.motif_agg_min;
+        p.agg_words = (m > 0 && p.agg_min > 0) ? mt_agg_words(m) : 0;
+        p.npat = m > 0 ? npat : 0;
+        const size_t mt_bytes = ((sizeof(MtWarp) + 15) & ~size_t(15)) + sizeof(unsigned long long) * ((p.npat + 1) & ~1) +
+                                4 * (size_t)((p.agg_words + 3) & ~3) + p.mark_stride + 4 * (size_t)p.slab_ints;
+        p.warp_bytes = (int)((p.cq_words * 4 + mt_bytes + 15) & ~size_t(15));
+        return (size_t)wpb * p.warp_bytes;
+    };
+    // (the limit on the graphs' sizes is the walk's, whichever way motifs are counted)
+    size_t smem = layout(hom_k);
     if (smem > 227 * 1024) fail(GPM_ENOTIMPL, "batched state does not fit in shared memory (graphs too large)");
+    if (hom) smem = layout(0);
     GPM_CUDA(cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = resident_blocks((const void*)k_batch, wpb * 32, smem);
     if (per_sm <= 0) fail(GPM_EINVAL, "batched kernel cannot be resident with this configuration");
@@ -349,7 +365,9 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     const size_t G = (size_t)b->n_graphs;
     const size_t ctl_words = (sizeof(Control) + 7) / 8;
     c.words = G + G * npat + ctl_words;
+    const size_t hom_bytes = sizeof(unsigned long long) * (G * HOM_N + 1);
     try {
+        if (hom) c.dev_hom.ensure(hom_bytes);
         c.dev_out.ensure(sizeof(unsigned long long) * c.words);
         GPM_CUDA(cudaMallocHost(&c.host_out, sizeof(unsigned long long) * c.words));
     } catch (...) {
@@ -361,6 +379,29 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     p.ctl = reinterpret_cast<Control*>(p.motif_out + G * npat);
     c.blocks = blocks;
     c.wpb = wpb;
+    c.launches = (n_units > 0 ? 1 : 0) + (hom ? 2 : 0);
+    HomLaunch hp{};
+    Grid hgr;
+    if (hom) {
+        hp.indptr = p.indptr;
+        hp.indices = p.indices;
+        hp.deg = g->degree.as<int32_t>();
+        hp.goff = p.goff;
+        hp.vgraph = p.vgraph;
+        hp.n = g->n;
+        hp.grab = 16;     // neighbouring vertices: mostly one graph
+        hp.maxn = b->max_graph_n;
+        hp.maxd = std::max(g->max_deg, 1);
+        hp.hom = c.dev_hom.as<unsigned long long>();
+        hp.ticket = hp.hom + G * HOM_N;
+        hp.ctl = p.ctl;
+        hgr = plan_hom(hp, hom_k, g->num_sms);
+        device_hom_table(hom_k);
+        if (n_units == 0) {
+            c.blocks = hgr.blocks;
+            c.wpb = hgr.warps_per_block;
+        }
+    }
 
     cudaGraph_t graph = nullptr;
     GPM_CUDA(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
@@ -368,6 +409,11 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     if (e1 == cudaSuccess && p.n_units > 0) {
         k_batch<<<blocks, wpb * 32, smem, b->stream>>>(p);
         e1 = cudaGetLastError();
+    }
+    if (e1 == cudaSuccess && hom) {
+        e1 = cudaMemsetAsync(c.dev_hom.ptr, 0, hom_bytes, b->stream);
+        if (e1 == cudaSuccess) e1 = launch_hom(hp, hom_k, hgr, b->stream);
+        if (e1 == cudaSuccess) e1 = launch_hom_finish(hp.hom, b->n_graphs, hom_k, p.motif_out, b->stream);
     }
     if (e1 == cudaSuccess)
         e1 = cudaMemcpyAsync(c.host_out, c.dev_out.ptr, sizeof(unsigned long long) * c.words, cudaMemcpyDeviceToHost,
@@ -510,7 +556,7 @@ void batch_count(gpm_batch* b, int kc, int km, uint64_t* clique_counts, uint64_t
     st.kernel_ms = ms;
     st.units_done = h->units_done;
     st.busy_warp_ns = h->busy_ns;
-    st.kernel_launches = 1;
+    st.kernel_launches = cap.launches;
     st.grid_blocks = cap.blocks;
     st.warps_per_block = cap.wpb;
     b->stats = st;

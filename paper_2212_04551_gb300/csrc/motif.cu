@@ -18,6 +18,7 @@
 #include "common.cuh"
 #include "monitor.cuh"
 #include "motif_dev.cuh"
+#include "motif_hom.cuh"
 #include "list_ring.cuh"
 
 namespace gpm {
@@ -310,6 +311,14 @@ void run_motif(gpm_graph* g, int k, const int32_t* d_roots, int64_t n_roots,
     const PatternTable& tab = pattern_table(k);
     const int npat = (int)tab.num_patterns;
     cudaStream_t s = g->stream;
+    // Whole-graph counts of small patterns come from homomorphism counts
+    // (motif_hom.cu); lists of roots, schedules, per-root results, listing and
+    // monitored runs are defined on the walk, and so is motif_agg_min = 0.
+    if (!d_roots && !plan && !d_per_root && !monitored && !list && g->cfg.motif_agg_min > 0 &&
+        hom_applies(g->n, g->max_deg, k)) {
+        run_motif_hom(g, k, counts_out);
+        return;
+    }
     if (!d_roots) {
         d_roots = ensure_root_order(g, GPM_APP_MOTIF);
         n_roots = g->n;

@@ -1,0 +1,65 @@
+// motif_hom.cuh -- induced motif counts of k = 3 .. 5 vertices from
+// homomorphism counts (shared by motif_hom.cu and the batched launch).
+#pragma once
+
+#include "common.cuh"
+
+namespace gpm {
+
+// The connected graphs on at most five vertices, by the sums that count their
+// homomorphisms into G (edges 1-2, 1-3, ...: see hom_edges() in motif_hom.cu).
+enum Hom {
+    // d^a s^b T^c summed over the vertices u: d = degree of u, s = sum of its
+    // neighbours' degrees, T = twice its triangles
+    H_POINT, H_EDGE, H_CHERRY, H_TRI, H_STAR3, H_PATH4, H_PAW, H_STAR4, H_PATH5, H_FORK, H_CRICKET, H_LOLLI, H_BOWTIE,
+    H_UNIFORM,                         // their number
+    // the rest: sums over pairs and triples of vertices
+    H_CYCLE4 = H_UNIFORM, H_DIAMOND, H_K4, H_CYCLE5, H_BANNER, H_BULL, H_K23, H_DART, H_KITE, H_HOUSE, H_GEM, H_BOOK,
+    H_K4TAIL, H_SPOKE, H_WHEEL, H_K5P3, H_K5E, H_K5, HOM_N
+};
+
+// Counts of size k from the sums: pattern p occurs
+// (sum_j coef[p * HOM_N + j] hom[j]) / aut[p] times (wrapping 64-bit sums, the
+// result of which is exact: every homomorphism count is below 2^63).
+struct HomTable {
+    int k = 0, npat = 0;
+    std::vector<long long> coef;
+    std::vector<long long> aut;
+};
+const HomTable& hom_table(int k);                 // host, built once per k
+const long long* device_hom_table(int k);         // coef, then aut; uploaded once per device
+
+struct HomLaunch {
+    const int32_t* __restrict__ indptr;
+    const int32_t* __restrict__ indices;
+    const int32_t* __restrict__ deg;
+    const int32_t* __restrict__ order;    // the order vertices are taken in (nullptr: by id)
+    const int32_t* __restrict__ goff;     // batch: vertex range of every graph (nullptr: one graph)
+    const int32_t* __restrict__ vgraph;   // batch: graph of every vertex
+    long long n;
+    int grab;                             // vertices a warp takes at a time
+    int maxn;                             // vertices of the largest graph
+    int maxd;                             // largest degree
+    int warp_words;                       // shared words per warp
+    unsigned long long* hom;              // [graph][HOM_N], zero
+    unsigned long long* ticket;           // next vertex, zero
+    Control* ctl;
+};
+
+constexpr int HOM_WARPS = 4;              // warps per block
+constexpr int HOM_MAX_N = 16384;          // vertices of one graph (shared-memory arrays over them)
+constexpr int HOM_MAX_D = 1024;           // largest degree (bit rows over a neighbourhood)
+
+// Whether graphs of at most n vertices and degree d are counted this way.
+bool hom_applies(long long n, long long d, int k);
+int hom_warp_words(int n, int d, int k);
+// Fills warp_words and sizes the launch (no stream operations); the launch itself (nothing
+// throws between the two ends of a capture).
+Grid plan_hom(HomLaunch& p, int k, int sms);
+cudaError_t launch_hom(const HomLaunch& p, int k, const Grid& gr, cudaStream_t s);
+// Whole-graph counts of g where hom_applies (stats filled)
+void run_motif_hom(gpm_graph* g, int k, uint64_t* counts_out);
+// out[g * npat + p] = count of pattern p in graph g
+cudaError_t launch_hom_finish(const unsigned long long* hom, int n_graphs, int k, unsigned long long* out, cudaStream_t s);
+
+}  // namespace gpm
