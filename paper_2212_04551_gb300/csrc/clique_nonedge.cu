@@ -70,6 +70,7 @@ struct NeLaunch {
     int maxd, w, ws;                      // heavy: largest d, its words, the row stride (odd)
     int warp_words;                       // heavy: shared words per warp
     unsigned int* next_child;             // heavy: per position, the next child not yet taken
+    unsigned int* tri;                    // nullable: triangles per out-list entry (rounds = 0)
     NeParams ne;
     Control* ctl;
     unsigned long long* ticket;           // next position (light) or root offer (heavy)
@@ -169,6 +170,11 @@ __global__ void __launch_bounds__(NE_LIGHT_WARPS * 32) k_clique_ne_light(NeLaunc
                         if (lo < d && W.list[lo] == x) {
                             atomicOr(&W.g[i], 1u << lo);
                             atomicOr(&W.g[lo], 1u << i);
+                            if (p.tri) {
+                                atomicAdd(&p.tri[beg + i], 1u);
+                                atomicAdd(&p.tri[beg + lo], 1u);
+                                atomicAdd(&p.tri[b + t + z], 1u);
+                            }
                         }
                     }
                 }
@@ -505,6 +511,11 @@ __global__ void __launch_bounds__(NE_WARPS * 32) k_clique_ne_heavy(NeLaunch p) {
                         const int px = pos[lo];
                         atomicOr(&rows[pi * p.ws + (px >> 5)], 1u << (px & 31));
                         atomicOr(&rows[px * p.ws + (pi >> 5)], 1u << (pi & 31));
+                        if (p.tri) {
+                            atomicAdd(&p.tri[beg + i], 1u);
+                            atomicAdd(&p.tri[beg + lo], 1u);
+                            atomicAdd(&p.tri[b + t + z], 1u);
+                        }
                     }
                 }
             }
@@ -578,7 +589,7 @@ static const unsigned long long* device_binomials() {
 // Whole-graph clique counts of sizes k_lo .. k_hi (k_hi >= 3) into ctl (its
 // counters zero); roots above the bitmap limit are left out.  Returns the
 // number of launches; grid/warps of the larger one for the statistics.
-int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* grid) {
+int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* grid, unsigned int* tri) {
     cudaStream_t s = g->stream;
     NeLaunch p{};
     p.roots = ensure_root_order(g, GPM_APP_CLIQUE);
@@ -590,6 +601,7 @@ int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* 
     p.ne.k_hi = k_hi;
     p.ne.binom = device_binomials();
     p.ctl = ctl;
+    p.tri = tri;
     // positions by out-degree: [0, above) list path, [above, big) heavy, [big, all) light
     const int need = std::max(p.ne.k_lo - 1, 1);
     const long long above = roots_at_least(g, NE_BINOM_N + 1);

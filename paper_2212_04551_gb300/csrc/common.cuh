@@ -211,8 +211,10 @@ void run_clique_dfs(gpm_graph* g, int k, uint64_t* count_out);   // the paper's 
 void run_clique_list(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_t n_roots,
                      unsigned long long* d_per_root, Control* ctl, int bitmap_limit);
 // clique_nonedge.cu: whole-graph counts of sizes k_lo .. k_hi (k_hi >= 3) into
-// ctl, without the roots above the bitmap limit; returns the launches made
-int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* grid);
+// ctl, without the roots above the bitmap limit; returns the launches made.
+// tri (nullable, k_hi <= 5): per entry of the orientation's out-lists, += the
+// triangles on that edge.
+int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* grid, unsigned int* tri = nullptr);
 void run_motif_monitored(gpm_graph* g, int k, double threshold, uint64_t* counts_out, MonitorStats* ms);
 
 // clique.cu / motif.cu

@@ -312,12 +312,17 @@ void run_motif(gpm_graph* g, int k, const int32_t* d_roots, int64_t n_roots,
     const int npat = (int)tab.num_patterns;
     cudaStream_t s = g->stream;
     // Whole-graph counts of small patterns come from homomorphism counts
-    // (motif_hom.cu); lists of roots, schedules, per-root results, listing and
+    // (motif_hom.cu, motif_sparse.cu); lists of roots, schedules, per-root results, listing and
     // monitored runs are defined on the walk, and so is motif_agg_min = 0.
-    if (!d_roots && !plan && !d_per_root && !monitored && !list && g->cfg.motif_agg_min > 0 &&
-        hom_applies(g->n, g->max_deg, k)) {
-        run_motif_hom(g, k, counts_out);
-        return;
+    if (!d_roots && !plan && !d_per_root && !monitored && !list && g->cfg.motif_agg_min > 0) {
+        if (hom_applies(g->n, g->max_deg, k)) {
+            run_motif_hom(g, k, counts_out);
+            return;
+        }
+        if (motif_sparse_applies(g, k)) {
+            run_motif_sparse(g, k, counts_out);
+            return;
+        }
     }
     if (!d_roots) {
         d_roots = ensure_root_order(g, GPM_APP_MOTIF);

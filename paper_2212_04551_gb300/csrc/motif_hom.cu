@@ -396,9 +396,13 @@ void run_motif_hom(gpm_graph* g, int k, uint64_t* counts_out) {
     st.grid_blocks = gr.blocks;
     st.warps_per_block = gr.warps_per_block;
     g->stats = st;
+    hom_combine(t, h.hom, counts_out);
+}
+
+void hom_combine(const HomTable& t, const unsigned long long* hom, uint64_t* counts_out) {
     for (int q = 0; q < t.npat; q++) {
         unsigned long long sum = 0;
-        for (int j = 0; j < HOM_N; j++) sum += (unsigned long long)t.coef[(size_t)q * HOM_N + j] * h.hom[j];
+        for (int j = 0; j < HOM_N; j++) sum += (unsigned long long)t.coef[(size_t)q * HOM_N + j] * hom[j];
         counts_out[q] = sum / (unsigned long long)t.aut[q];
     }
 }

@@ -27,6 +27,7 @@ struct HomTable {
     std::vector<long long> aut;
 };
 const HomTable& hom_table(int k);                 // host, built once per k
+void hom_combine(const HomTable& t, const unsigned long long* hom, uint64_t* counts_out);
 const long long* device_hom_table(int k);         // coef, then aut; uploaded once per device
 
 struct HomLaunch {
@@ -59,6 +60,9 @@ Grid plan_hom(HomLaunch& p, int k, int sms);
 cudaError_t launch_hom(const HomLaunch& p, int k, const Grid& gr, cudaStream_t s);
 // Whole-graph counts of g where hom_applies (stats filled)
 void run_motif_hom(gpm_graph* g, int k, uint64_t* counts_out);
+// Larger graphs, k = 3 and 4 (motif_sparse.cu; builds the orientation)
+bool motif_sparse_applies(gpm_graph* g, int k);
+void run_motif_sparse(gpm_graph* g, int k, uint64_t* counts_out);
 // out[g * npat + p] = count of pattern p in graph g
 cudaError_t launch_hom_finish(const unsigned long long* hom, int n_graphs, int k, unsigned long long* out, cudaStream_t s);
 

@@ -57,3 +57,29 @@ def test_degree_limit(leaves):
         got = _by_code(dg, k)
         assert sum(got.values()) == comb(leaves, k - 1) and len(got) == 2
         assert max(got.values()) == comb(leaves, k - 1) - comb(leaves - 2, k - 3)
+
+
+def _random_edges(n, m, seed):
+    rng = np.random.default_rng(seed)
+    return G.from_edges(n, rng.integers(0, n, m), rng.integers(0, n, m))
+
+
+SPARSE = {
+    "rmat15": lambda: G.rmat(15, 8, 0.57, 0.19, 0.19, 3),
+    "rmat15_any_order": lambda: G.relabel(G.rmat(15, 4, 0.57, 0.19, 0.19, 4), np.random.default_rng(1).permutation(1 << 15)),
+    "hub": lambda: G.disjoint_union(G.star(1500), G.gnp(60, 0.5, 2), G.turan(50, 2), G.empty(7)),
+    "above_16_bit_ids": lambda: _random_edges(70001, 200000, 5),
+    "global_counters": lambda: G.disjoint_union(_random_edges(115001, 250000, 6), G.complete(40), G.turan(90, 3)),
+}
+
+
+@pytest.mark.parametrize("name", SPARSE)
+@pytest.mark.parametrize("k", [3, 4])
+def test_larger_graphs_against_the_walk(name, k):
+    """Graphs beyond the per-vertex arrays (motif_sparse.cu)."""
+    g = SPARSE[name]()
+    dg = gpm.graph_from_csr(g)
+    ours = gpm.gpm_motif_count(dg, k)
+    assert gpm.gpm_get_stats(dg)["kernel_launches"] >= 2
+    gpm.gpm_set_config(dg, motif_agg_min=0)
+    assert np.array_equal(ours, gpm.gpm_motif_count(dg, k))
