@@ -188,7 +188,7 @@ __global__ void __maxnreg__(96) k_clique(CliqueParams p) {
             }
             if (p.donate && !registered) {
                 int ok = 0;
-                if (lane == 0) ok = gpm_idle_register(p.ring_seq, p.ring_ids, p.ring_cap, &ctl->q_tail, gw) ? 1 : 0;
+                if (lane == 0) ok = gpm_idle_register(p.ring_seq, p.ring_ids, p.ring_cap, ctl, gw) ? 1 : 0;
                 registered = __shfl_sync(GPM_FULL_MASK, ok, 0) != 0;
             }
             // the termination state is shared by every idle warp: look at it

@@ -1056,11 +1056,7 @@ __device__ bool cq_walk(const CliqueWalk& a, const CliqueUnit* unit, int root_po
             int err = 0, want = 0;
             if (lane == 0) {
                 err = *(volatile int*)&ctl->error;
-                if (now - t_start > a.donate_after_ns) {
-                    const unsigned long long qh = *(volatile unsigned long long*)&ctl->q_head;
-                    const unsigned long long qt = *(volatile unsigned long long*)&ctl->q_tail;
-                    want = qt > qh;   // a registered idle warp is waiting
-                }
+                if (now - t_start > a.donate_after_ns) want = gpm_idle_waiting(ctl);
             }
             err = __shfl_sync(GPM_FULL_MASK, err, 0);
             if (err) return false;
@@ -1078,7 +1074,7 @@ __device__ bool cq_walk(const CliqueWalk& a, const CliqueUnit* unit, int root_po
                     if (mid < 0) break;
                     if (lane == 0) {
                         int wid;
-                        if (gpm_idle_claim(a.ring_seq, a.ring_ids, a.ring_cap, &ctl->q_head, &wid)) {
+                        if (gpm_idle_claim(a.ring_seq, a.ring_ids, a.ring_cap, ctl, &wid)) {
                             unsigned char* box = a.mbox + (size_t)wid * a.mbox_stride;
                             CliqueUnit* dst = reinterpret_cast<CliqueUnit*>(box + sizeof(MailHdr));
                             CliqueUnit u;

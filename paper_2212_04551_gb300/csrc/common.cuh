@@ -139,7 +139,7 @@ struct alignas(128) Control {
     int error;                        // GPM_* status raised on the device
     int stop;                         // host-monitored balancing: spill the remaining work and leave
     alignas(128) int active;          // host-monitored balancing: warps holding a unit
-    int pad_active;
+    int idle;                         // hand-offs: registered idle warps not yet claimed (busy warps look here)
     unsigned long long spill_n;       // host-monitored balancing: units spilled so far
     alignas(128) unsigned long long q_head;   // (alignas binds per declarator: one per line)
     unsigned long long q_tail;
@@ -323,14 +323,16 @@ __device__ __forceinline__ void gpm_atomic_add_cc(unsigned long long* c, unsigne
 
 // ------------------------------------------------- donation queue (device)
 //
-// Bounded multi-producer multi-consumer ring of sequence-numbered slots
-// (after D. Vyukov's bounded MPMC queue).  Slot i starts with seq = i.  A
-// producer reserves position p (seq == p), writes the unit -- and any payload
-// kept beside the ring at index p % cap -- and publishes seq = p + 1.  A
-// consumer claims p (seq == p + 1), reads, and releases with seq = p + cap.
-// Every loop is bounded: a full, empty or contended queue reports failure
-// and the caller keeps (or goes on looking for) work.  Reads of published
-// data go through L2 (ld.global.cg): L1 is not coherent across SMs.
+// Ring of sequence-numbered slots between idle warps and donors.  Slot i
+// starts with seq = i; the warp that holds position p for writing waits for
+// seq == p, writes and publishes seq = p + 1; the one that holds it for
+// reading waits for that, reads and releases with seq = p + cap.  Positions
+// are handed out by one atomic add each -- `idle` counts the published ids not
+// yet spoken for, so that a donor takes a position only if an id is, or is
+// about to be, there.  (Handing them out by compare-and-swap let one donor
+// through per round trip to L2, about 10^6 hand-offs a second however many
+// warps waited.)  Every wait is bounded.  Reads of published data go through
+// L2 (ld.global.cg): L1 is not coherent across SMs.
 struct QSeq {
     unsigned long long seq;
 };
@@ -344,59 +346,13 @@ __global__ void k_validate(const int32_t* __restrict__ indptr, const int32_t* __
 __global__ void k_indptr_monotone(const int32_t* __restrict__ indptr, int32_t n, int* __restrict__ bad);
 }
 
-__device__ __forceinline__ bool gpm_q_reserve(QSeq* q, unsigned long long cap, unsigned long long* tail,
-                                              unsigned long long* out_pos) {
-    unsigned long long pos = *(volatile unsigned long long*)tail;
-    for (int tries = 0; tries < 256; tries++) {
-        const unsigned long long seq = *(volatile unsigned long long*)&q[pos % cap].seq;
-        const long long dif = (long long)(seq - pos);
-        if (dif == 0) {
-            const unsigned long long prev = atomicCAS(tail, pos, pos + 1);
-            if (prev == pos) {
-                *out_pos = pos;
-                return true;
-            }
-            pos = prev;
-        } else if (dif < 0) {
-            return false;  // full
-        } else {
-            pos = *(volatile unsigned long long*)tail;
-        }
-    }
+constexpr int GPM_Q_SPINS = 1 << 16;
+
+__device__ __forceinline__ bool gpm_q_await(QSeq* q, unsigned long long cap, unsigned long long pos,
+                                            unsigned long long seq) {
+    for (int tries = 0; tries < GPM_Q_SPINS; tries++)
+        if (*(volatile unsigned long long*)&q[pos % cap].seq == seq) return true;
     return false;
-}
-
-// call after every writer of the slot's data has executed __threadfence()
-__device__ __forceinline__ void gpm_q_publish(QSeq* q, unsigned long long cap, unsigned long long pos) {
-    atomicExch(&q[pos % cap].seq, pos + 1);
-}
-
-__device__ __forceinline__ bool gpm_q_claim(QSeq* q, unsigned long long cap, unsigned long long* head,
-                                            unsigned long long* out_pos) {
-    unsigned long long pos = *(volatile unsigned long long*)head;
-    for (int tries = 0; tries < 256; tries++) {
-        const unsigned long long seq = *(volatile unsigned long long*)&q[pos % cap].seq;
-        const long long dif = (long long)(seq - (pos + 1));
-        if (dif == 0) {
-            const unsigned long long prev = atomicCAS(head, pos, pos + 1);
-            if (prev == pos) {
-                __threadfence();
-                *out_pos = pos;
-                return true;
-            }
-            pos = prev;
-        } else if (dif < 0) {
-            return false;  // empty
-        } else {
-            pos = *(volatile unsigned long long*)head;
-        }
-    }
-    return false;
-}
-
-// call after every reader of the slot's data is done (and fenced)
-__device__ __forceinline__ void gpm_q_release(QSeq* q, unsigned long long cap, unsigned long long pos) {
-    atomicExch(&q[pos % cap].seq, pos + cap);
 }
 
 // ------------------------------------------ direct hand-off of donated work
@@ -412,23 +368,33 @@ struct MailHdr {
     int pad[3];
 };
 
-__device__ __forceinline__ bool gpm_idle_register(QSeq* seq, int32_t* ids, unsigned long long cap,
-                                                  unsigned long long* tail, int wid) {
-    unsigned long long pos;
-    if (!gpm_q_reserve(seq, cap, tail, &pos)) return false;
+__device__ __forceinline__ bool gpm_idle_register(QSeq* seq, int32_t* ids, unsigned long long cap, gpm::Control* ctl,
+                                                  int wid) {
+    const unsigned long long pos = atomicAdd(&ctl->q_tail, 1ull);
+    if (!gpm_q_await(seq, cap, pos, pos)) return false;   // never: the ring holds every warp
     ids[pos % cap] = wid;
     __threadfence();
-    gpm_q_publish(seq, cap, pos);
+    atomicExch(&seq[pos % cap].seq, pos + 1);
+    __threadfence();
+    atomicAdd(&ctl->idle, 1);
     return true;
 }
 
-__device__ __forceinline__ bool gpm_idle_claim(QSeq* seq, int32_t* ids, unsigned long long cap,
-                                               unsigned long long* head, int* wid) {
-    unsigned long long pos;
-    if (!gpm_q_claim(seq, cap, head, &pos)) return false;
+// a registered idle warp waits (a look, nothing claimed)
+__device__ __forceinline__ bool gpm_idle_waiting(const gpm::Control* ctl) { return *(volatile int*)&ctl->idle > 0; }
+
+__device__ __forceinline__ bool gpm_idle_claim(QSeq* seq, int32_t* ids, unsigned long long cap, gpm::Control* ctl,
+                                               int* wid) {
+    if (atomicSub(&ctl->idle, 1) <= 0) {
+        atomicAdd(&ctl->idle, 1);
+        return false;
+    }
+    const unsigned long long pos = atomicAdd(&ctl->q_head, 1ull);
+    if (!gpm_q_await(seq, cap, pos, pos + 1)) return false;   // never: published before it was counted
+    __threadfence();
     *wid = __ldcg(ids + pos % cap);
     __threadfence();
-    gpm_q_release(seq, cap, pos);
+    atomicExch(&seq[pos % cap].seq, pos + cap);
     return true;
 }
 

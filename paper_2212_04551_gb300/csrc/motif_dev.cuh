@@ -35,7 +35,15 @@ constexpr int MT_MAXK = GPM_MOTIF_MAX_K;
 constexpr int MT_MAXPAT = 853;                 // connected 7-vertex patterns: per-block shared counters
 constexpr int MT_MAXPAT8 = 11117;              // connected 8-vertex patterns: counted in global memory
 constexpr unsigned long long MT_CHECK_NS = 4000;  // busy warps look for idle ones at most this often
-constexpr float MT_MIN_DONATE_WORK = 2048.f;    // estimated leaves a handed-over range must carry
+// A handed-over range must be worth the replay of its path: this many adjacency
+// entries scanned, by the estimate of mt_donate -- MT_ENTRIES per child of a
+// node one level above the leaves, MT_NODE for the pushes and pops of such a
+// node.  Per-root 5-motifs of rmat12 at 512 / 2,048 / 8,192 / 32,768 entries:
+// 92 / 84 / 84 / 86 ms; 7-motifs of G(500, 1500): 6.1 / 7.0 / 29 / 111 ms.
+constexpr float MT_MIN_DONATE_WORK = 2048.f;
+constexpr float MT_ENTRIES = 32.f;
+constexpr float MT_NODE = 512.f;
+constexpr int MT_MIN_LEFT = (int)(4 * MT_MIN_DONATE_WORK / MT_ENTRIES);   // children that always make such a range
 constexpr int MT_AGG_UNROLL = 4;                 // adjacency entries per lane per round (mt_tail_agg)
 
 // A work unit: the children at positions [lo, hi) of the extension array of
@@ -341,12 +349,15 @@ __device__ __noinline__ static void mt_donate(Control* ctl, QSeq* ring_seq, int3
         if (to - from < max(donate_min, 2)) continue;
         const int len = W->len[t];
         const int mid = mt_split(from, to, len, k - 1 - t);
-        // estimated work of the later part: sum of (len - c)^e, e = levels below
-        const float q = (float)(k - t);
-        const float est = (__powf((float)(len - mid), q) - __powf(fmaxf((float)(len - to), 1.0f), q)) / q;
+        // estimated work of the later part: the children one level above the
+        // leaves (sum of (len - c)^e, e = levels in between), each of which scans
+        // an adjacency list, and the nodes above these children
+        const float q = (float)(k - 1 - t), A = (float)(len - mid), B = fmaxf((float)(len - to), 1.0f);
+        float est = MT_ENTRIES * (__powf(A, q) - __powf(B, q)) / q;
+        if (q > 1.f) est += MT_NODE * (__powf(A, q - 1.f) - __powf(B, q - 1.f)) / (q - 1.f);
         if (est < MT_MIN_DONATE_WORK) continue;
         int wid;
-        if (!gpm_idle_claim(ring_seq, ring_ids, ring_cap, &ctl->q_head, &wid)) return;
+        if (!gpm_idle_claim(ring_seq, ring_ids, ring_cap, ctl, &wid)) return;
         if (wid < 0 || (unsigned long long)wid >= ring_cap) {   // never: ids are registered warps
             atomicCAS(&ctl->error, 0, DEV_ECHECK + 4);
             return;
@@ -370,53 +381,75 @@ __device__ __noinline__ static void mt_donate(Control* ctl, QSeq* ring_seq, int3
     }
 }
 
+// First position in the sorted N(v) holding a vertex above `root`, for one lane
+// alone: three probes per step, issued together, so that a list of 1,024
+// entries takes five rounds of dependent loads instead of ten.
+__device__ __forceinline__ int mt_above_lane(const int32_t* __restrict__ indices, int lo, int hi, int root) {
+    while (hi - lo > 3) {                    // indices[lo - 1] <= root < indices[hi], where these exist
+        const int q = (hi - lo) >> 2;
+        const int p1 = lo + q, p2 = lo + 2 * q, p3 = lo + 3 * q;
+        const bool b1 = indices[p1] <= root, b2 = indices[p2] <= root, b3 = indices[p3] <= root;
+        lo = b3 ? p3 + 1 : b2 ? p2 + 1 : b1 ? p1 + 1 : lo;
+        hi = !b1 ? p1 : !b2 ? p2 : !b3 ? p3 : hi;
+    }
+    while (lo < hi && indices[lo] <= root) lo++;
+    return lo;
+}
+
 // The last two levels below a node tr of size k-2 (level l = k-2, array ext
 // of length L), counted by class instead of leaf by leaf.  Its children are
-// w = ext[c], c in A = [cur, hi); child w is the (k-1)-set tr+w, and its
-// k-vertex leaves are tr+w+x for every later entry x = ext[c'] (c' > c) and
-// for every exclusive neighbour x of w (above the root, neither in tr nor
-// adjacent to it).  The induced graph of a leaf is fixed by code(tr), the
-// class of w and of x -- an entry's class is its adjacency to tr, mark bits
-// 0 .. k-3 -- and whether w and x are adjacent.  So:
+// w = ext[c], c in [cur, hi); child w is the (k-1)-set tr+w, and its k-vertex
+// leaves are tr+w+x for every later entry x = ext[c'] (c' > c) and for every
+// exclusive neighbour x of w (above the root, neither in tr nor adjacent to
+// it).  The induced graph of a leaf is fixed by code(tr), the class of w and
+// of x -- an entry's class is its adjacency to tr, mark bits 0 .. k-3 -- and
+// whether w and x are adjacent.  So, with A the children done and B the
+// entries after them:
 //
-//   * pairs {w, x} of entries: with HA / HB the class histograms of A and of
-//     B = [hi, L), the pairs of classes {s1, s2} number C(HA[s],2) (s1 = s2)
-//     or HA[s1] HA[s2] within A, plus HA[s1] HB[s2] (+ HA[s2] HB[s1]) across;
-//     of these, the adjacent ones are found by scanning N(w) for every w in A
-//     (an entry x of A counted from its smaller endpoint only, an entry of B
-//     always), and the rest are non-adjacent;
+//   * pairs {w, x} of entries: with HA / HB the class histograms of A and B,
+//     the pairs of classes {s1, s2} number C(HA[s],2) (s1 = s2) or
+//     HA[s1] HA[s2] within A, plus HA[s1] HB[s2] (+ HA[s2] HB[s1]) across; of
+//     these, the adjacent ones are found by scanning N(w) for every w in A,
+//     and the rest are non-adjacent;
 //   * exclusive neighbours: counted per class of w during the same scans.
 //
 // One scan of N(w) per child replaces the per-leaf walk over the later
-// entries (quadratic in L).  Mark bits 6 and 5 flag the entries of A u B and
-// of B during the call (free at this level: tr uses bits 0 .. k-3 and 7).
-// The adjacency lists of 32 children at a time are scanned as one flattened
-// range, so every lane has an entry whatever the degrees.
-template <class Sink>
+// entries (quadratic in L).  Children are done 32 at a time, their adjacency
+// lists scanned as one flattened range, so that every lane has an entry
+// whatever the degrees.  During the call mark bit 6 flags the entries not done
+// yet and bit 5 those of the current 32 (free at this level: tr uses bits
+// 0 .. k-3 and 7): an adjacent entry counts if it is not done, and within the
+// 32 from its smaller endpoint.  The counts are then those of the children
+// done, after any 32 of them, so a call with DONATE leaves early (cur moved on
+// to the first child not done) when an idle warp waits for a hand-off: below a
+// hub one call scans 10^5 entries, milliseconds in which nothing could be
+// handed over (rmat12 5-motifs per root: see k_motif in motif.cu).
+template <bool DONATE, class Sink>
 __device__ __noinline__ void mt_tail_agg(const MotifWalk& a, MtWarp* W, int l, const int32_t* ext, int root,
                                          Sink& sink, unsigned long long& leaves, unsigned long long& scanned,
-                                         int lane) {
+                                         unsigned long long t_start, unsigned long long& last_check, int lane) {
     const int C = 1 << l;                        // classes: adjacency to tr[0 .. l-1]
     const unsigned lowtr = (unsigned)C - 1u;
-    const int a0 = W->cur[l], a1 = W->hi[l], L = W->len[l];
+    const int a0 = W->cur[l], L = W->len[l];
+    int a1 = W->hi[l];
     uint32_t* HA = a.agg;
-    uint32_t* HB = HA + C;
-    uint32_t* E = HB + C;
+    uint32_t* H = HA + C;                        // of A and B together
+    uint32_t* E = H + C;
     uint32_t* P = E + C;                         // P[s1 * C + s2], s1 <= s2
     for (int i = lane; i < 3 * C + C * C; i += 32) HA[i] = 0u;
     __syncwarp();
-    // classes of A and B, and their range marks
+    // classes of all entries, and their marks
     for (int j0 = a0; j0 < L; j0 += 32) {
         const int j = j0 + lane;
         int key = -1;
         if (j < L) {
             const int x = ext[j];
             const unsigned char m = a.mk[x - a.mbase];
-            a.mk[x - a.mbase] = m | (unsigned char)(j < a1 ? 0x40 : 0x60);
-            key = (int)(m & lowtr) + (j < a1 ? 0 : C);
+            a.mk[x - a.mbase] = m | (unsigned char)0x40;
+            key = (int)(m & lowtr);
         }
         const unsigned grp = __match_any_sync(GPM_FULL_MASK, key);
-        if (key >= 0 && lane == __ffs(grp) - 1) HA[key] += (uint32_t)__popc(grp);
+        if (key >= 0 && lane == __ffs(grp) - 1) H[key] += (uint32_t)__popc(grp);
     }
     __syncwarp();
     // scan N(w) for the children, 32 at a time
@@ -425,15 +458,18 @@ __device__ __noinline__ void mt_tail_agg(const MotifWalk& a, MtWarp* W, int l, c
         int w = 0, sw = 0, b = 0, e = 0;
         if (c < a1) {
             w = ext[c];
-            sw = a.mk[w - a.mbase] & lowtr;
-            int lo = a.indptr[w], hi = a.indptr[w + 1];
-            e = hi;
-            while (lo < hi) {                    // first neighbour above the root
-                const int mid = (lo + hi) >> 1;
-                if (a.indices[mid] <= root) lo = mid + 1; else hi = mid;
-            }
-            b = lo;
+            const unsigned char m = a.mk[w - a.mbase];
+            sw = m & lowtr;
+            a.mk[w - a.mbase] = m | (unsigned char)0x20;
+            e = a.indptr[w + 1];
+            b = mt_above_lane(a.indices, a.indptr[w], e, root);
         }
+        {
+            const int key = c < a1 ? sw : -1;
+            const unsigned grp = __match_any_sync(GPM_FULL_MASK, key);
+            if (key >= 0 && lane == __ffs(grp) - 1) HA[key] += (uint32_t)__popc(grp);
+        }
+        __syncwarp();
         const int len = e - b;
         int incl = len;
 #pragma unroll
@@ -473,7 +509,7 @@ __device__ __noinline__ void mt_tail_agg(const MotifWalk& a, MtWarp* W, int l, c
                     const unsigned m = ms[u];
                     if ((m & (lowtr | 0x80u)) == 0) {
                         ex = true;                   // exclusive neighbour of w
-                    } else if ((m & 0x40u) && ((m & 0x20u) || xs[u] > wts[u])) {
+                    } else if ((m & 0x40u) && (!(m & 0x20u) || xs[u] > wts[u])) {
                         const int s2 = (int)(m & lowtr);   // adjacent pair of entries (rare)
                         atomicAdd(&P[min(sts[u], s2) * C + max(sts[u], s2)], 1u);
                     }
@@ -493,8 +529,24 @@ __device__ __noinline__ void mt_tail_agg(const MotifWalk& a, MtWarp* W, int l, c
                 }
             }
         }
+        // these children are done
+        __syncwarp();
+        if (c < a1) a.mk[w - a.mbase] &= (unsigned char)0x9f;
+        __syncwarp();
+        // (leave only with enough left for a hand-off of MT_MIN_DONATE_WORK, and
+        // after an eighth of the entries: a later call looks at them all again)
+        if (DONATE && a1 - (c0 + 32) >= MT_MIN_LEFT && (c0 + 32 - a0) * 8 >= L - a0) {
+            int stop = 0;
+            if (lane == 0) {
+                const unsigned long long now = gpm_globaltimer();
+                if (now - last_check >= MT_CHECK_NS && now - t_start > a.donate_after_ns) {
+                    stop = gpm_idle_waiting(a.ctl) || *(volatile int*)&a.ctl->error;
+                    if (!stop) last_check = now;
+                }
+            }
+            if (__shfl_sync(GPM_FULL_MASK, stop, 0)) a1 = c0 + 32;
+        }
     }
-    __syncwarp();
     // patterns: w = v_l (bits at mt_code_off(l), none for l = 1), x = v_{l+1}
     const int codetr = l >= 2 ? W->code[l] : 0;
     const int offx = mt_code_off(l + 1);
@@ -502,7 +554,7 @@ __device__ __noinline__ void mt_tail_agg(const MotifWalk& a, MtWarp* W, int l, c
     for (int idx = lane; idx < C * C; idx += 32) {
         const int s1 = idx >> l, s2 = idx & (C - 1);
         if (s1 > s2) continue;
-        const unsigned long long ha1 = HA[s1], ha2 = HA[s2], hb1 = HB[s1], hb2 = HB[s2];
+        const unsigned long long ha1 = HA[s1], ha2 = HA[s2], hb1 = H[s1] - ha1, hb2 = H[s2] - ha2;
         const unsigned long long within = s1 == s2 ? ha1 * (ha1 - (ha1 ? 1 : 0)) / 2 : ha1 * ha2;
         const unsigned long long across = ha1 * hb2 + (s1 != s2 ? ha2 * hb1 : 0ull);
         const unsigned long long adj = P[idx];
@@ -530,8 +582,8 @@ __device__ __noinline__ void mt_tail_agg(const MotifWalk& a, MtWarp* W, int l, c
         mine += E[s1];
     }
     leaves += mine;
-    // drop the range marks
-    for (int j = a0 + lane; j < L; j += 32) a.mk[ext[j] - a.mbase] &= (unsigned char)0x9f;
+    // drop the marks of the entries after them
+    for (int j = a1 + lane; j < L; j += 32) a.mk[ext[j] - a.mbase] &= (unsigned char)0x9f;
     __syncwarp();
     if (lane == 0) W->cur[l] = a1;
     __syncwarp();
@@ -597,6 +649,7 @@ __device__ __forceinline__ bool mt_walk(const MotifWalk& a, MtWarp* W, int pdept
     unsigned long long last_check = t_start;   // lane 0
     for (;;) {
         const int c = W->cur[l];
+        bool tail = false;
         if (c >= W->hi[l]) {
             if (l == pdepth) break;
             // pop tr[l-1] (pushed at depth l-1)
@@ -614,63 +667,65 @@ __device__ __forceinline__ bool mt_walk(const MotifWalk& a, MtWarp* W, int pdept
         const int32_t* ext = l == pdepth ? unit_ext : a.slab + a.lvl_off[l];
         if (l + 2 == k && a.agg_min > 0 && W->len[l] - c >= a.agg_min) {
             // one level above the leaves with many entries left: count the
-            // remaining children's leaves by class (then pop)
+            // remaining children's leaves by class (then pop, or hand some over)
             __syncwarp();
-            mt_tail_agg(a, W, l, ext, root, sink, unit_leaves, scanned, lane);
-            continue;
+            mt_tail_agg<DONATE>(a, W, l, ext, root, sink, unit_leaves, scanned, t_start, last_check, lane);
+            tail = true;
         }
-        const int w = ext[c];
-        __syncwarp();                       // every lane has read cur[l] before it moves on
-        if (lane == 0) W->cur[l] = c + 1;
-        const int codew = mt_child_code(a, W, l, w);
-        const int wb = mt_above(a.indptr, a.indices, w, root, lane), we = a.indptr[w + 1];
-        if (lane == 0 && l + 1 != k - 1) scanned += (unsigned)(we - wb);
-        const unsigned char low = (unsigned char)(0x80 | ((1u << l) - 1));
-        if (l + 1 == k - 1) {
-            if constexpr (Sink::kList) {
-                // ---- last level, listing: a record per leaf of tr + w
-                mt_list_leaves(a, W, l, c, ext, w, wb, we, codew, sink, unit_leaves, lane);
-            } else {
-                // ---- last level: leaves of the (k-1)-set tr + w
-                const int offk = mt_code_off(l + 1);
-                if (lane == 0) scanned += 2ull * (unsigned)(we - wb);
-                int excl = 0;
-                for (int t = wb + lane; t < we; t += 32) {
-                    const int x = a.indices[t];
-                    const unsigned char m = a.mk[x - a.mbase];
-                    excl += (m & low) == 0 ? 1 : 0;
-                    a.mk[x - a.mbase] = m | (unsigned char)(1u << l);
-                }
-                excl = __reduce_add_sync(GPM_FULL_MASK, (unsigned)excl);
-                __syncwarp();
-                if (excl && lane == 0) {
-                    const int pid = a.lut[codew | ((1 << l) << offk)];
-                    if (pid == 0xffff) atomicExch(a.err, DEV_EINVAL);
-                    else sink.add(pid, (unsigned long long)excl);
-                    unit_leaves += (unsigned)excl;
-                }
-                const int len = W->len[l];
-                const unsigned lowk = (1u << (l + 1)) - 1u;
-                for (int j0 = c + 1; j0 < len; j0 += 32) {
-                    const int j = j0 + lane;
-                    const bool act = j < len;
-                    int pid = 0;
-                    if (act) {
-                        const int x = ext[j];
-                        const int sig = a.mk[x - a.mbase] & lowk;
-                        pid = a.lut[codew | (sig << offk)];
-                        unit_leaves++;
+        if (!tail) {
+            const int w = ext[c];
+            __syncwarp();                       // every lane has read cur[l] before it moves on
+            if (lane == 0) W->cur[l] = c + 1;
+            const int codew = mt_child_code(a, W, l, w);
+            const int wb = mt_above(a.indptr, a.indices, w, root, lane), we = a.indptr[w + 1];
+            if (lane == 0 && l + 1 != k - 1) scanned += (unsigned)(we - wb);
+            const unsigned char low = (unsigned char)(0x80 | ((1u << l) - 1));
+            if (l + 1 == k - 1) {
+                if constexpr (Sink::kList) {
+                    // ---- last level, listing: a record per leaf of tr + w
+                    mt_list_leaves(a, W, l, c, ext, w, wb, we, codew, sink, unit_leaves, lane);
+                } else {
+                    // ---- last level: leaves of the (k-1)-set tr + w
+                    const int offk = mt_code_off(l + 1);
+                    if (lane == 0) scanned += 2ull * (unsigned)(we - wb);
+                    int excl = 0;
+                    for (int t = wb + lane; t < we; t += 32) {
+                        const int x = a.indices[t];
+                        const unsigned char m = a.mk[x - a.mbase];
+                        excl += (m & low) == 0 ? 1 : 0;
+                        a.mk[x - a.mbase] = m | (unsigned char)(1u << l);
                     }
-                    mt_count_leaves(sink, act, pid, a.err);
+                    excl = __reduce_add_sync(GPM_FULL_MASK, (unsigned)excl);
+                    __syncwarp();
+                    if (excl && lane == 0) {
+                        const int pid = a.lut[codew | ((1 << l) << offk)];
+                        if (pid == 0xffff) atomicExch(a.err, DEV_EINVAL);
+                        else sink.add(pid, (unsigned long long)excl);
+                        unit_leaves += (unsigned)excl;
+                    }
+                    const int len = W->len[l];
+                    const unsigned lowk = (1u << (l + 1)) - 1u;
+                    for (int j0 = c + 1; j0 < len; j0 += 32) {
+                        const int j = j0 + lane;
+                        const bool act = j < len;
+                        int pid = 0;
+                        if (act) {
+                            const int x = ext[j];
+                            const int sig = a.mk[x - a.mbase] & lowk;
+                            pid = a.lut[codew | (sig << offk)];
+                            unit_leaves++;
+                        }
+                        mt_count_leaves(sink, act, pid, a.err);
+                    }
+                    __syncwarp();
+                    for (int t = wb + lane; t < we; t += 32) a.mk[a.indices[t] - a.mbase] &= (unsigned char)~(1u << l);
+                    __syncwarp();
                 }
-                __syncwarp();
-                for (int t = wb + lane; t < we; t += 32) a.mk[a.indices[t] - a.mbase] &= (unsigned char)~(1u << l);
-                __syncwarp();
+            } else {
+                // ---- push w: ext_{l+1} = ext_l[c+1:] ++ exclusive neighbours of w
+                if (!mt_push(a, W, l, c, ext, w, wb, we, codew, lane)) return false;
+                l++;
             }
-        } else {
-            // ---- push w: ext_{l+1} = ext_l[c+1:] ++ exclusive neighbours of w
-            if (!mt_push(a, W, l, c, ext, w, wb, we, codew, lane)) return false;
-            l++;
         }
 
         if (!DONATE && a.monitor) {
@@ -720,11 +775,7 @@ __device__ __forceinline__ bool mt_walk(const MotifWalk& a, MtWarp* W, int pdept
             if (lane == 0 && now - last_check >= MT_CHECK_NS) {
                 last_check = now;
                 err = *(volatile int*)&ctl->error;
-                if (now - t_start > a.donate_after_ns) {
-                    const unsigned long long qh = *(volatile unsigned long long*)&ctl->q_head;
-                    const unsigned long long qt = *(volatile unsigned long long*)&ctl->q_tail;
-                    want = qt > qh;   // a registered idle warp is waiting
-                }
+                if (now - t_start > a.donate_after_ns) want = gpm_idle_waiting(ctl);
             }
             err = __shfl_sync(GPM_FULL_MASK, err, 0);
             if (err) return false;

@@ -44,6 +44,7 @@ def test_against_the_walk(name, k):
     ours = gpm.gpm_motif_count(dg, k)
     st = gpm.gpm_get_stats(dg)
     assert st["units_done"] == g.n and st["kernel_launches"] == 1
+    assert np.array_equal(ours, gpm.gpm_count_roots(dg, gpm.GPM_APP_MOTIF, k)[0])
     gpm.gpm_set_config(dg, motif_agg_min=0)
     assert np.array_equal(ours, gpm.gpm_motif_count(dg, k))
 
@@ -81,5 +82,6 @@ def test_larger_graphs_against_the_walk(name, k):
     dg = gpm.graph_from_csr(g)
     ours = gpm.gpm_motif_count(dg, k)
     assert gpm.gpm_get_stats(dg)["kernel_launches"] >= 2
+    assert np.array_equal(ours, gpm.gpm_count_roots(dg, gpm.GPM_APP_MOTIF, k)[0])
     gpm.gpm_set_config(dg, motif_agg_min=0)
     assert np.array_equal(ours, gpm.gpm_motif_count(dg, k))
