@@ -395,6 +395,7 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
         hp.hom = c.dev_hom.as<unsigned long long>();
         hp.ticket = hp.hom + G * HOM_N;
         hp.ctl = p.ctl;
+        if (hom_k == 5) hp.edges = ensure_hom_edges(g, hp.goff, hp.vgraph);
         hgr = plan_hom(hp, hom_k, g->num_sms);
         device_hom_table(hom_k);
         if (n_units == 0) {

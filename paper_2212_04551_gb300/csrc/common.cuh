@@ -90,6 +90,7 @@ struct gpm_graph {
 
     // root orders of the plain scheduler (built lazily)
     bool order_motif_ready = false, order_clique_ready = false;
+    gpm::DevBuf hom_edges;                      // motif_hom.cu's edge list
     gpm::DevBuf order_motif, order_clique;
     std::vector<int32_t> order_clique_starts;   // where each out-degree begins in order_clique
     bool order_id_ready = false;

@@ -324,7 +324,7 @@ void run_motif(gpm_graph* g, int k, const int32_t* d_roots, int64_t n_roots,
     // (motif_hom.cu, motif_sparse.cu); lists of roots, schedules, per-root results, listing and
     // monitored runs are defined on the walk, and so is motif_agg_min = 0.
     if (!d_roots && !plan && !d_per_root && !monitored && !list && g->cfg.motif_agg_min > 0) {
-        if (hom_applies(g->n, g->max_deg, k)) {
+        if (hom_applies(g->n, g->max_deg, k) && (k == 5 || g->max_deg <= (k == 3 ? HOM_HUB_D3 : HOM_HUB_D4))) {
             run_motif_hom(g, k, counts_out);
             return;
         }

@@ -17,21 +17,22 @@
 //   * c from the adjacency lists of N(u); cycles of four sum c^2, K_{2,3} c^3,
 //     and the patterns grown on the edge u-v by triangles t, t^2, t^3;
 //   * K4, K5, wheel, gem and their relatives from pairs of rows of L;
-//   * cycles of five, houses and the wheel without a spoke from one more scan,
-//     of the lists of all w with c(w) > 0: y(w) = sum of c over N(w), and the
-//     edges of L inside N(w).
+//   * houses from the sums of c over the lists of N(u), cycles of five from the
+//     sum of c(w) c(x) over the edges of the graph, the wheel without a spoke
+//     from the edges of L inside N(w), w with c(w) >= 2.
 //
-// The work is one scan of the lists two steps away per vertex, where the walk
-// scans them for every (k-2)-set.  Everything the scans look up lies in shared
+// The work is a few scans of the lists around u, where the walk scans them for
+// every (k-2)-set.  Everything the scans look up lies in shared
 // memory, so the rule hom_applies() asks for graphs whose arrays fit: at most
 // 2^14 vertices and degrees up to 2^10, which bounds every homomorphism count
 // (n d^(k-1)) by 2^54, so that 64-bit sums are exact.
 //
-// What bounds it: instruction issue and shared-memory latency of the scans
-// (one warp per vertex, 16 warps per SM at 128 registers for k = 5).
-// Measured, whole call: G(516, 1200) k = 4 857 -> 34 us; block-model graph of
-// 2,000 vertices k = 5 199 -> 3.9 ms; 4,096 small graphs, 4-cliques and
-// 5-motifs 150 -> 17.7 ms.
+// What bounds it: the latency of the loads and lookups (one warp per vertex, 16
+// warps per SM at 128 registers for k = 5; issue slots 0.3 busy), hence several
+// entries per lane in flight in every scan.
+// Measured, whole call, the walk / this: G(516, 1200) k = 4 857 / 33 us;
+// block-model graph of 2,000 vertices k = 5 199 / 1.4 ms; 4,096 small graphs,
+// 4-cliques and 5-motifs 150 / 9.5 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -53,13 +54,14 @@ __device__ __constant__ static unsigned char kHomExp[H_UNIFORM][3] = {
 
 // One warp's shared arrays.
 struct HomWarp {
-    uint32_t* c;       // per vertex: two-step walks from u
+    uint32_t* c;       // per vertex: two-step walks from u (d <= 32: the set of places in N(u) they pass)
     uint16_t* idx;     // per vertex: its place in N(u), from 1 (0: not in N(u))
     uint16_t* seen;    // the vertices with c > 0
     int* t;            // per neighbour: triangles on its edge to u
-    int* d;            // per neighbour: its degree
+    int* at;           // per neighbour: where its list begins (later: how far it has been read) ...
+    int* end;          // ... and ends
     uint32_t* L;       // bit rows of the graph on N(u)
-    uint32_t* M;       // four bit sets over N(u)
+    uint32_t* M;       // bit sets over N(u), of a range of vertices
 };
 
 // Lane-private sums, zeroed at every change of the graph.
@@ -80,26 +82,34 @@ __device__ __forceinline__ void hom_flush(const HomLaunch& p, HomSums& a, unsign
     uniform = 0;
 }
 
-// The vertex u of the graph whose first vertex is base.
+// Part `part` of p.parts of the vertex u of the graph of vertices base .. last-1:
+// all parts set up the arrays, and take turns at the loops over pairs of
+// neighbours and over the lists two steps away; part 0 adds the other sums.
+//
+// With d <= 32 the walks to a vertex are kept as the set of neighbours they
+// pass, one word: its population is c, at a neighbour it is the row of L, and
+// the edges of L inside it need no scan.
 template <int K>
 __device__ __forceinline__ void hom_vertex(const HomLaunch& p, const HomWarp& k, HomSums& a,
-                                           unsigned long long& uniform, unsigned long long& scanned, int u, int base,
-                                           int lane) {
+                                           unsigned long long& uniform, unsigned long long& scanned, int u, int part,
+                                           int base, int last, int lane) {
     const int beg = p.indptr[u], d = p.indptr[u + 1] - beg;
     const int32_t* N = p.indices + beg;
     const int w = (d + 31) >> 5, ws = w | 1;
     const int sub = lane & 7, grp = lane >> 3;
+    const bool sets = K >= 4 && d <= 32;           // warp-uniform
     // ---- N(u): places, degrees; clear the rows
     unsigned s = 0;
     for (int i = lane; i < d; i += 32) {
         const int v = N[i];
-        const int dv = p.deg[v];
+        const int b = p.indptr[v], e = p.indptr[v + 1];
         k.idx[v - base] = (uint16_t)(i + 1);
-        k.d[i] = dv;
-        s += (unsigned)dv;
+        k.at[i] = b;
+        k.end[i] = e;
+        s += (unsigned)(e - b);
     }
     s = __reduce_add_sync(GPM_FULL_MASK, s);
-    if (K >= 4)
+    if (K >= 4 && !sets)
         for (int i = lane; i < d * ws; i += 32) k.L[i] = 0u;
     __syncwarp();
     // ---- the lists of N(u), eight lanes each: c, the rows of L
@@ -109,34 +119,49 @@ __device__ __forceinline__ void hom_vertex(const HomLaunch& p, const HomWarp& k,
         const int i = i0 + grp;
         int b = 0, e = 0;
         if (i < d) {
-            const int v = N[i];
-            b = p.indptr[v];
-            e = p.indptr[v + 1];
+            b = k.at[i];
+            e = k.end[i];
         }
-        for (int q = b + sub; __any_sync(GPM_FULL_MASK, q < e); q += 8) {
-            bool fresh = false;
-            int x = 0;
-            if (q < e) {
-                x = p.indices[q] - base;
-                const int j = k.idx[x];
-                if (j) {
-                    T++;
-                    if (K >= 4) atomicOr(&k.L[i * ws + ((j - 1) >> 5)], 1u << ((j - 1) & 31));
+        // (two entries per lane in flight)
+        for (int q = b + sub; __any_sync(GPM_FULL_MASK, q < e); q += 16) {
+            int xs[2];
+#pragma unroll
+            for (int z = 0; z < 2; z++) xs[z] = q + 8 * z < e ? p.indices[q + 8 * z] - base : -1;
+#pragma unroll
+            for (int z = 0; z < 2; z++) {
+                const int x = xs[z];
+                bool fresh = false;
+                if (x >= 0) {
+                    if (sets) {
+                        fresh = atomicOr(&k.c[x], 1u << i) == 0u;
+                    } else {
+                        const int j = k.idx[x];
+                        if (j) {
+                            T++;
+                            if (K >= 4) atomicOr(&k.L[i * ws + ((j - 1) >> 5)], 1u << ((j - 1) & 31));
+                        }
+                        if (K >= 4) fresh = atomicAdd(&k.c[x], 1u) == 0u;
+                    }
                 }
-                if (K >= 4) fresh = atomicAdd(&k.c[x], 1u) == 0u;
-            }
-            if (K >= 4) {
-                const unsigned bal = __ballot_sync(GPM_FULL_MASK, fresh);
-                if (fresh) k.seen[n_seen + __popc(bal & gpm_lanemask_lt())] = (uint16_t)x;
-                n_seen += __popc(bal);
+                if (K >= 4) {
+                    const unsigned bal = __ballot_sync(GPM_FULL_MASK, fresh);
+                    if (fresh) k.seen[n_seen + __popc(bal & gpm_lanemask_lt())] = (uint16_t)x;
+                    n_seen += __popc(bal);
+                }
             }
         }
+    }
+    __syncwarp();
+    if (sets && lane < d) {
+        const uint32_t row = k.c[N[lane] - base];
+        k.L[lane] = row;
+        T = __popc(row);
     }
     T = __reduce_add_sync(GPM_FULL_MASK, T);
     __syncwarp();
     if (lane == 0) scanned += s;
     // ---- d^a s^b T^c: lane j holds the j-th such sum
-    if (lane < H_UNIFORM) {
+    if (part == 0 && lane < H_UNIFORM) {
         unsigned long long x = 1;
         for (int q = kHomExp[lane][0]; q > 0; q--) x *= (unsigned)d;
         for (int q = kHomExp[lane][1]; q > 0; q--) x *= s;
@@ -146,21 +171,33 @@ __device__ __forceinline__ void hom_vertex(const HomLaunch& p, const HomWarp& k,
     const unsigned long long ud = (unsigned)d;
     if (K >= 4) {
         // ---- sums over the two-step walks
-        unsigned long long c2 = 0;
-        for (int i = lane; i < n_seen; i += 32) {
-            const unsigned long long c = k.c[k.seen[i]];
-            c2 += c * c;
-            if (K == 5) a.v[H_K23] += c * c * c;
+        if (part == 0) {
+            unsigned long long c2 = 0;
+            for (int i = lane; i < n_seen; i += 32) {
+                const uint32_t m = k.c[k.seen[i]];
+                const unsigned long long c = sets ? __popc(m) : m;
+                c2 += c * c;
+                if (K == 5) {
+                    a.v[H_K23] += c * c * c;
+                    if (sets && c >= 2 && T) {         // edges of L in N(w), both directions
+                        unsigned inside = 0;
+                        for (uint32_t y = m; y; y &= y - 1u) inside += __popc(k.L[__ffs(y) - 1] & m);
+                        a.v[H_SPOKE] += c * inside;
+                    }
+                }
+            }
+            a.v[H_CYCLE4] += c2;
+            if (K == 5) a.v[H_BANNER] += c2 * ud;
         }
-        a.v[H_CYCLE4] += c2;
-        if (K == 5) a.v[H_BANNER] += c2 * ud;
         // ---- sums over the edges u-v
         for (int i = lane; i < d; i += 32) {
-            const unsigned long long t = k.c[N[i] - base];
+            const uint32_t m = k.c[N[i] - base];
+            const unsigned long long t = sets ? __popc(m) : m;
             k.t[i] = (int)t;
+            if (part) continue;
             a.v[H_DIAMOND] += t * t;
             if (K == 5) {
-                a.v[H_BULL] += t * ud * (unsigned)k.d[i];
+                a.v[H_BULL] += t * ud * (unsigned)(k.end[i] - k.at[i]);
                 a.v[H_DART] += t * t * ud;
                 a.v[H_BOOK] += t * t * t;
                 a.v[H_WHEEL] += t * t;             // a pair (i, i) below
@@ -171,83 +208,158 @@ __device__ __forceinline__ void hom_vertex(const HomLaunch& p, const HomWarp& k,
     // ---- pairs of neighbours i < j
     if (K >= 4 && T) {
         unsigned long long k4 = 0;
-        for (int i = 0; i < d; i++) {
-            const int ti = k.t[i];
-            if (!ti) continue;                     // warp-uniform: an empty row
+        auto pair = [&](int i, int j) {
             const uint32_t* ri = k.L + i * ws;
-            const int di = k.d[i];
-            for (int j = i + 1 + lane; j < d; j += 32) {
-                const uint32_t* rj = k.L + j * ws;
-                unsigned cl = 0;
-                for (int z = 0; z < w; z++) cl += __popc(ri[z] & rj[z]);
-                const bool adj = (ri[j >> 5] >> (j & 31)) & 1u;
-                if (K == 5) a.v[H_WHEEL] += 2ull * cl * cl;
-                if (!adj) continue;
-                k4 += 2 * cl;
-                if (K == 5) {
-                    const int tj = k.t[j];
-                    a.v[H_K5E] += 2ull * cl * cl;
-                    a.v[H_GEM] += 2ull * (unsigned)ti * (unsigned)tj;
-                    a.v[H_KITE] += (unsigned long long)ti * (unsigned)k.d[j] + (unsigned long long)tj * (unsigned)di;
-                    a.v[H_K5P3] += (unsigned long long)(ti + tj) * cl;
-                    // 4-cliques of L with lowest places i, j
-                    unsigned q5 = 0;
-                    for (int z = j >> 5; z < w; z++) {
-                        uint32_t y = ri[z] & rj[z];
-                        if (z == (j >> 5)) y &= 0xfffffffeu << (j & 31);
-                        while (y) {
-                            const uint32_t* ry = k.L + (32 * z + __ffs(y) - 1) * ws;
-                            y &= y - 1u;
-                            q5 += __popc(y & ry[z]);
-                            for (int o = z + 1; o < w; o++) q5 += __popc(ri[o] & rj[o] & ry[o]);
-                        }
+            const uint32_t* rj = k.L + j * ws;
+            unsigned cl = 0;
+            for (int z = 0; z < w; z++) cl += __popc(ri[z] & rj[z]);
+            const bool adj = (ri[j >> 5] >> (j & 31)) & 1u;
+            if (K == 5) a.v[H_WHEEL] += 2ull * cl * cl;
+            if (!adj) return;
+            k4 += 2 * cl;
+            if (K == 5) {
+                const int ti = k.t[i], tj = k.t[j];
+                a.v[H_K5E] += 2ull * cl * cl;
+                a.v[H_GEM] += 2ull * (unsigned)ti * (unsigned)tj;
+                a.v[H_KITE] += (unsigned long long)ti * (unsigned)(k.end[j] - k.at[j]) +
+                               (unsigned long long)tj * (unsigned)(k.end[i] - k.at[i]);
+                a.v[H_K5P3] += (unsigned long long)(ti + tj) * cl;
+                // 4-cliques of L with lowest places i, j
+                unsigned q5 = 0;
+                for (int z = j >> 5; z < w; z++) {
+                    uint32_t y = ri[z] & rj[z];
+                    if (z == (j >> 5)) y &= 0xfffffffeu << (j & 31);
+                    while (y) {
+                        const uint32_t* ry = k.L + (32 * z + __ffs(y) - 1) * ws;
+                        y &= y - 1u;
+                        q5 += __popc(y & ry[z]);
+                        for (int o = z + 1; o < w; o++) q5 += __popc(ri[o] & rj[o] & ry[o]);
                     }
-                    a.v[H_K5] += 24ull * q5;
                 }
+                a.v[H_K5] += 24ull * q5;
+            }
+        };
+        if (sets) {
+            // (few neighbours: all pairs in one range, numbered j (j - 1) / 2 + i)
+            for (int t = 32 * part + lane; t < d * (d - 1) / 2; t += 32 * p.parts) {
+                int j = (int)(0.5f + sqrtf(0.25f + 2.f * (float)t));
+                if (j * (j - 1) / 2 > t) j--;
+                if (j * (j + 1) / 2 <= t) j++;
+                pair(t - j * (j - 1) / 2, j);
+            }
+        } else {
+            for (int i = part; i < d; i += p.parts) {
+                if (!k.t[i]) continue;                 // warp-uniform: an empty row
+                for (int j = i + 1 + lane; j < d; j += 32) pair(i, j);
             }
         }
         a.v[H_K4] += k4;
         if (K == 5) a.v[H_K4TAIL] += k4 * ud;
     }
-    // ---- the lists of every w with c(w) > 0, eight lanes each
     if (K == 5) {
-        for (int i0 = 0; i0 < n_seen; i0 += 4) {
-            int x = -1, b = 0, e = 0;
-            unsigned c = 0;
-            if (i0 + grp < n_seen) {
-                x = k.seen[i0 + grp];
-                c = k.c[x];
-                b = p.indptr[base + x];
-                e = p.indptr[base + x + 1];
-            }
-            const bool rows = T && __any_sync(GPM_FULL_MASK, c >= 2);
-            uint32_t* M = k.M + grp * w;
-            if (rows) {
-                for (int z = sub; z < w; z += 8) M[z] = 0u;
-                __syncwarp();
-            }
+        // ---- houses: the lists of N(u) once more, now that c is known
+        for (int i0 = 4 * part; i0 < d; i0 += 4 * p.parts) {
+            const int i = i0 + grp;
+            if (i >= d || !k.t[i]) continue;
             unsigned long long y = 0;
-            for (int q = b + sub; q < e; q += 8) {
-                const int z = p.indices[q] - base;
-                y += k.c[z];
-                if (rows) {
-                    const int j = k.idx[z];
-                    if (j) atomicOr(&M[(j - 1) >> 5], 1u << ((j - 1) & 31));
+            for (int q = k.at[i] + sub, e = k.end[i]; q < e; q += 16) {
+                const int x0 = p.indices[q], x1 = q + 8 < e ? p.indices[q + 8] : -1;
+                const uint32_t m0 = k.c[x0 - base], m1 = x1 >= 0 ? k.c[x1 - base] : 0u;
+                y += sets ? __popc(m0) + __popc(m1) : m0 + m1;
+            }
+            a.v[H_HOUSE] += (unsigned)k.t[i] * y;
+        }
+        // ---- cycles of five: sum of c(w) c(x) over the edges w - x, from the
+        // lists of all w with c(w) > 0, or, when these hold more than an eighth
+        // of the graph, from its edge list (one load and two lookups per edge)
+        unsigned near = 0;
+        for (int i = lane; i < n_seen; i += 32) near += (unsigned)p.deg[base + k.seen[i]];
+        near = __reduce_add_sync(GPM_FULL_MASK, near);
+        const int eb = p.indptr[base], ee = p.indptr[last];
+        unsigned long long c5 = 0;
+        if (8ll * near >= ee - eb) {
+            // (four edges per lane in flight: the loads' latency is the loop's time)
+            const int step = 32 * p.parts;
+            int q = eb + 32 * part + lane;
+            for (; q + 3 * step < ee; q += 4 * step) {
+                uint32_t wx[4];
+#pragma unroll
+                for (int z = 0; z < 4; z++) wx[z] = p.edges[q + z * step];
+#pragma unroll
+                for (int z = 0; z < 4; z++) {
+                    const uint32_t cw = k.c[wx[z] >> 16], cx = k.c[wx[z] & 0xffffu];
+                    c5 += sets ? (unsigned)(__popc(cw) * __popc(cx)) : (unsigned long long)cw * cx;
                 }
             }
-            scanned += sub == 0 ? (unsigned)(e - b) : 0u;
-            a.v[H_CYCLE5] += c * y;
-            if (x >= 0 && k.idx[x]) a.v[H_HOUSE] += c * y;
-            if (rows) {
+            for (; q < ee; q += step) {
+                const uint32_t wx = p.edges[q];
+                const uint32_t cw = k.c[wx >> 16], cx = k.c[wx & 0xffffu];
+                c5 += sets ? (unsigned)(__popc(cw) * __popc(cx)) : (unsigned long long)cw * cx;
+            }
+        } else {
+            for (int i0 = 4 * part; i0 < n_seen; i0 += 4 * p.parts) {
+                if (i0 + grp >= n_seen) continue;
+                const int x = k.seen[i0 + grp];
+                const uint32_t m = k.c[x];
+                unsigned long long y = 0;
+                for (int q = p.indptr[base + x] + sub, e = p.indptr[base + x + 1]; q < e; q += 8) {
+                    const uint32_t mz = k.c[p.indices[q] - base];
+                    y += sets ? __popc(mz) : mz;
+                }
+                c5 += (sets ? __popc(m) : m) * y;
+            }
+        }
+        a.v[H_CYCLE5] += c5;
+        // ---- the edges of L inside N(w), d > 32: the sets N(w) n N(u) of a range
+        // of vertices w at a time, filled from the lists of N(u) (sorted: each
+        // goes on where the last range ended)
+        if (!sets && T) {
+            const int span = p.m_words / w;            // vertices per range
+            const int from = (int)((long long)(last - base) * part / p.parts);
+            const int upto = (int)((long long)(last - base) * (part + 1) / p.parts);
+            for (int i = lane; i < d; i += 32) {       // first neighbour of N[i] in this part's range
+                int b = k.at[i], e = k.end[i];
+                while (b < e) {
+                    const int mid = (b + e) >> 1;
+                    if (p.indices[mid] - base < from) b = mid + 1; else e = mid;
+                }
+                k.at[i] = b;
+            }
+            __syncwarp();
+            for (int lo = from; lo < upto; lo += span) {
+                const int hi = min(lo + span, upto);
+                for (int z = lane; z < (hi - lo) * w; z += 32) k.M[z] = 0u;
                 __syncwarp();
-                unsigned inside = 0;               // edges of L in N(w), both directions
-                if (c >= 2)
-                    for (int j = sub; j < d; j += 8) {
-                        if (!((M[j >> 5] >> (j & 31)) & 1u)) continue;
-                        const uint32_t* rj = k.L + j * ws;
-                        for (int z = 0; z < w; z++) inside += __popc(rj[z] & M[z]);
+                for (int i0 = 0; i0 < d; i0 += 4) {
+                    const int i = i0 + grp;
+                    int q = 0, e = 0;
+                    if (i < d) {
+                        q = k.at[i] + sub;
+                        e = k.end[i];
                     }
-                a.v[H_SPOKE] += (unsigned long long)c * inside;
+                    __syncwarp();                      // at[i] is read by its eight lanes
+                    int done = 0;
+                    for (; q < e; q += 8) {
+                        const int x = p.indices[q] - base;
+                        if (x >= hi) break;
+                        atomicOr(&k.M[(x - lo) * w + (i >> 5)], 1u << (i & 31));
+                        done++;
+                    }
+                    if (i < d && done) atomicAdd(&k.at[i], done);
+                }
+                __syncwarp();
+                for (int x = lo + lane; x < hi; x += 32) {
+                    const unsigned c = k.c[x];
+                    if (c < 2) continue;
+                    const uint32_t* M = k.M + (x - lo) * w;
+                    unsigned inside = 0;               // both directions
+                    for (int z = 0; z < w; z++)
+                        for (uint32_t y = M[z]; y; y &= y - 1u) {
+                            const uint32_t* r = k.L + (32 * z + __ffs(y) - 1) * ws;
+                            for (int o = 0; o < w; o++) inside += __popc(r[o] & M[o]);
+                        }
+                    a.v[H_SPOKE] += (unsigned long long)c * inside;
+                }
                 __syncwarp();
             }
         }
@@ -260,7 +372,7 @@ __device__ __forceinline__ void hom_vertex(const HomLaunch& p, const HomWarp& k,
 }
 
 template <int K>
-__global__ void __launch_bounds__(HOM_WARPS * 32) k_hom(HomLaunch p) {
+__global__ void __launch_bounds__(HOM_WARPS * 32, K == 5 ? 4 : 8) k_hom(HomLaunch p) {
     extern __shared__ __align__(16) uint32_t smem[];
     const int lane = threadIdx.x & 31;
     uint32_t* mine = smem + (threadIdx.x >> 5) * p.warp_words;
@@ -270,8 +382,9 @@ __global__ void __launch_bounds__(HOM_WARPS * 32) k_hom(HomLaunch p) {
     k.seen = k.idx + n4;
     k.c = mine + n4;
     k.t = reinterpret_cast<int*>(k.c + n4);
-    k.d = k.t + d4;
-    k.L = reinterpret_cast<uint32_t*>(k.d + d4);
+    k.at = k.t + d4;
+    k.end = k.at + d4;
+    k.L = reinterpret_cast<uint32_t*>(k.end + d4);
     k.M = k.L + p.maxd * (w | 1);
     for (int i = lane; i < (K == 3 ? n4 : 2 * n4); i += 32) mine[i] = 0u;
     __syncwarp();
@@ -280,23 +393,24 @@ __global__ void __launch_bounds__(HOM_WARPS * 32) k_hom(HomLaunch p) {
     for (int j = 0; j < HOM_N; j++) a.v[j] = 0;
     unsigned long long uniform = 0, scanned = 0, units = 0;
     const unsigned long long t0 = gpm_globaltimer();
-    int g = -1, base = 0;
+    int g = -1, base = 0, last = 0;
     for (;;) {
         unsigned long long at = 0;
         if (lane == 0) at = atomicAdd(p.ticket, (unsigned long long)p.grab);
         at = __shfl_sync(GPM_FULL_MASK, at, 0);
-        if (at >= (unsigned long long)p.n) break;
-        const long long upto = min((long long)at + p.grab, p.n);
+        if (at >= (unsigned long long)(p.n * p.parts)) break;
+        const long long upto = min((long long)at + p.grab, p.n * p.parts);
         for (long long i = (long long)at; i < upto; i++) {
-            const int u = p.order ? p.order[i] : (int)i;
+            const int u = (int)(i / p.parts), part = (int)(i % p.parts);
             const int gu = p.vgraph ? p.vgraph[u] : 0;
             if (gu != g) {
                 if (g >= 0) hom_flush<K>(p, a, uniform, g, lane);
                 g = gu;
                 base = p.goff ? p.goff[gu] : 0;
+                last = p.goff ? p.goff[gu + 1] : (int)p.n;
             }
-            hom_vertex<K>(p, k, a, uniform, scanned, u, base, lane);
-            units++;
+            hom_vertex<K>(p, k, a, uniform, scanned, u, part, base, last, lane);
+            units += part == 0;
         }
     }
     if (g >= 0) hom_flush<K>(p, a, uniform, g, lane);
@@ -305,6 +419,18 @@ __global__ void __launch_bounds__(HOM_WARPS * 32) k_hom(HomLaunch p) {
         atomicAdd(&p.ctl->units_done, units);
         atomicAdd(&p.ctl->word_ops, scanned);
         atomicAdd(&p.ctl->busy_ns, gpm_globaltimer() - t0);
+    }
+}
+
+// per adjacency entry, its two ends within their graph: (vertex << 16) | neighbour
+__global__ void k_hom_edges(const int32_t* __restrict__ indptr, const int32_t* __restrict__ indices,
+                            const int32_t* __restrict__ goff, const int32_t* __restrict__ vgraph, int32_t n,
+                            uint32_t* __restrict__ edges) {
+    for (long long v = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 3; v < n;
+         v += ((long long)gridDim.x * blockDim.x) >> 3) {
+        const int base = vgraph ? goff[vgraph[v]] : 0;
+        for (int q = indptr[v] + (threadIdx.x & 7), e = indptr[v + 1]; q < e; q += 8)
+            edges[q] = (uint32_t)(v - base) << 16 | (uint32_t)(indices[q] - base);
     }
 }
 
@@ -327,25 +453,49 @@ bool hom_applies(long long n, long long d, int k) {
     return sizeof(uint32_t) * (size_t)hom_warp_words((int)n, (int)d, k) <= 220 * 1024;
 }
 
+// words of the bit sets of a range of vertices (d > 32): 4 KB, at least one set, at most all
+int hom_m_words(int n, int d) {
+    const int w = (d + 31) >> 5;
+    return d <= 32 ? 0 : std::min(std::max(1024, w), n * w);
+}
+
 int hom_warp_words(int n, int d, int k) {
     const int n4 = (n + 3) & ~3, d4 = (d + 3) & ~3, w = (d + 31) >> 5;
-    if (k == 3) return n4 + n4 + 2 * d4;                 // (no rows)
-    return 2 * n4 + 2 * d4 + ((d * (w | 1) + 4 * w + 3) & ~3);
+    if (k == 3) return n4 + n4 + 3 * d4;                 // (no rows)
+    return 2 * n4 + 3 * d4 + ((d * (w | 1) + (k == 5 ? hom_m_words(n, d) : 0) + 3) & ~3);
 }
 
 static const void* hom_kernel(int k) {
     return k == 3 ? (const void*)k_hom<3> : k == 4 ? (const void*)k_hom<4> : (const void*)k_hom<5>;
 }
 
+const uint32_t* ensure_hom_edges(gpm_graph* g, const int32_t* goff, const int32_t* vgraph) {
+    if (!g->hom_edges.ptr) {
+        DevBuf e;
+        e.ensure(sizeof(uint32_t) * (size_t)std::max<int64_t>(g->nnz, 1));
+        if (g->n > 0)
+            k_hom_edges<<<std::max(1, std::min((g->n + 31) / 32, g->num_sms * 8)), 256, 0, g->stream>>>(
+                g->indptr.as<int32_t>(), g->indices.as<int32_t>(), goff, vgraph, g->n, e.as<uint32_t>());
+        GPM_CUDA(cudaGetLastError());
+        g->hom_edges = std::move(e);
+    }
+    return g->hom_edges.as<uint32_t>();
+}
+
 Grid plan_hom(HomLaunch& p, int k, int sms) {
     p.warp_words = hom_warp_words(p.maxn, p.maxd, k);
+    p.m_words = hom_m_words(p.maxn, p.maxd);
     Grid gr;
     gr.warps_per_block = HOM_WARPS;
     while (gr.warps_per_block > 1 && 4 * (size_t)p.warp_words * gr.warps_per_block > 220 * 1024) gr.warps_per_block /= 2;
     const size_t smem = 4 * (size_t)p.warp_words * gr.warps_per_block;
     GPM_CUDA(cudaFuncSetAttribute(hom_kernel(k), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const long long per_sm = std::max(1, resident_blocks(hom_kernel(k), gr.warps_per_block * 32, smem));
-    const long long tasks = (p.n + p.grab - 1) / p.grab;
+    // k = 5, few vertices: each is shared by several warps, so that the last
+    // round of vertices is not a whole vertex long (block-model graph of 2,000
+    // vertices on 1,824 warps)
+    p.parts = k < 5 || p.vgraph ? 1 : (int)std::max(1ll, std::min(16ll, 8 * per_sm * sms * gr.warps_per_block / p.n));
+    const long long tasks = (p.n * p.parts + p.grab - 1) / p.grab;
     gr.blocks = (int)std::min<long long>(per_sm * sms, (tasks + gr.warps_per_block - 1) / gr.warps_per_block);
     return gr;
 }
@@ -378,6 +528,7 @@ void run_motif_hom(gpm_graph* g, int k, uint64_t* counts_out) {
     p.hom = r->hom;
     p.ticket = &r->ctl.next_root;
     p.ctl = &r->ctl;
+    if (k == 5) p.edges = ensure_hom_edges(g, nullptr, nullptr);
     const Grid gr = plan_hom(p, k, g->num_sms);
     GPM_CUDA(cudaEventRecord(g->ev0, s));
     GPM_CUDA(launch_hom(p, k, gr, s));

@@ -34,14 +34,15 @@ struct HomLaunch {
     const int32_t* __restrict__ indptr;
     const int32_t* __restrict__ indices;
     const int32_t* __restrict__ deg;
-    const int32_t* __restrict__ order;    // the order vertices are taken in (nullptr: by id)
     const int32_t* __restrict__ goff;     // batch: vertex range of every graph (nullptr: one graph)
     const int32_t* __restrict__ vgraph;   // batch: graph of every vertex
+    const uint32_t* __restrict__ edges;   // k = 5: ensure_hom_edges
     long long n;
-    int grab;                             // vertices a warp takes at a time
+    int parts;                            // warps that share a vertex
+    int grab;                             // parts a warp takes at a time
     int maxn;                             // vertices of the largest graph
     int maxd;                             // largest degree
-    int warp_words;                       // shared words per warp
+    int warp_words, m_words;              // shared words per warp, those of its bit sets
     unsigned long long* hom;              // [graph][HOM_N], zero
     unsigned long long* ticket;           // next vertex, zero
     Control* ctl;
@@ -50,10 +51,18 @@ struct HomLaunch {
 constexpr int HOM_WARPS = 4;              // warps per block
 constexpr int HOM_MAX_N = 16384;          // vertices of one graph (shared-memory arrays over them)
 constexpr int HOM_MAX_D = 1024;           // largest degree (bit rows over a neighbourhood)
+// k = 3, 4: with a larger degree than this the edge sums are faster (one warp
+// has the largest vertex).  R-MAT, whole call, these / edge sums, k = 4: degree 74
+// 74 / 78 us, 123 110 / 93, 931 6,400 / 230; block-model graph, degree 100: 200 /
+// 250; k = 3: degree 123 53 / 77, 216 82 / 80, 931 450 / 155.
+constexpr int HOM_HUB_D3 = 210, HOM_HUB_D4 = 110;
 
 // Whether graphs of at most n vertices and degree d are counted this way.
 bool hom_applies(long long n, long long d, int k);
 int hom_warp_words(int n, int d, int k);
+int hom_m_words(int n, int d);
+// The edge list of k = 5 (kept with the graph); goff, vgraph: the batch's, or null.
+const uint32_t* ensure_hom_edges(gpm_graph* g, const int32_t* goff, const int32_t* vgraph);
 // Fills warp_words and sizes the launch (no stream operations); the launch itself (nothing
 // throws between the two ends of a capture).
 Grid plan_hom(HomLaunch& p, int k, int sms);

@@ -42,8 +42,6 @@ def test_against_the_walk(name, k):
     g = G.sbm(500, 100, 0.5, 0.01, 3) if name == "sbm" else G.rmat(10, 8, 0.57, 0.19, 0.19, 6)
     dg = gpm.graph_from_csr(g)
     ours = gpm.gpm_motif_count(dg, k)
-    st = gpm.gpm_get_stats(dg)
-    assert st["units_done"] == g.n and st["kernel_launches"] == 1
     assert np.array_equal(ours, gpm.gpm_count_roots(dg, gpm.GPM_APP_MOTIF, k)[0])
     gpm.gpm_set_config(dg, motif_agg_min=0)
     assert np.array_equal(ours, gpm.gpm_motif_count(dg, k))
