@@ -19,6 +19,7 @@
 // The MLP is ~5k parameters and runs over at most a few hundred thousand
 // roots (~0.3 GFLOP): microseconds against seconds of enumeration, so it is
 // plain FP32 SIMT code with the weights broadcast from shared memory.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -39,71 +40,139 @@ static_assert(MLP_NPARAM == GPM_MLP_PARAMS, "parameter count");
 // ------------------------------------------------------------- features
 
 // triangles rooted at v in the degree orientation: sum over u in N+(v) of
-// |N+(v) & N+(u)| (binary search of N+(u)'s entries in N+(v)); warp per v
-__global__ void k_tri_root(const int32_t* __restrict__ off, const int32_t* __restrict__ adj,
-                           const int32_t* __restrict__ outdeg, int32_t n, float* __restrict__ tri) {
+// |N+(v) & N+(u)|.  Warp per v, eight lanes per list N+(u) with 16-byte loads
+// (the lists are padded and aligned for it), every entry searched in N+(v),
+// which lies in shared memory up to TRI_LIST entries.
+constexpr int TRI_LIST = 1024;
+constexpr int TRI_THREADS = 256;
+__global__ void __launch_bounds__(TRI_THREADS) k_tri_root(const int32_t* __restrict__ off,
+                                                          const int32_t* __restrict__ adj,
+                                                          const int32_t* __restrict__ outdeg, int32_t n,
+                                                          float* __restrict__ tri) {
+    __shared__ int32_t s_list[TRI_THREADS / 32][TRI_LIST];
     const int lane = threadIdx.x & 31;
+    int32_t* sl = s_list[threadIdx.x >> 5];
     const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     for (long long v = warp; v < n; v += nw) {
         const int b = off[v], d = outdeg[v];
+        const bool small = d <= TRI_LIST;
+        if (small)
+            for (int t = lane; t < d; t += 32) sl[t] = adj[b + t];
+        __syncwarp();
         long long c = 0;
-        for (int i = 0; i < d; i++) {
-            const int u = adj[b + i];
+        for (int i = lane >> 3; i < d; i += 4) {
+            const int u = small ? sl[i] : adj[b + i];
             const int ub = off[u], du = outdeg[u];
-            for (int t = lane; t < du; t += 32) {
-                const int x = adj[ub + t];
-                int lo = 0, hi = d - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (adj[b + mid] < x) lo = mid + 1; else hi = mid;
+            for (int t = 4 * (lane & 7); t < du; t += 32) {
+                const int4 x4 = *reinterpret_cast<const int4*>(adj + ub + t);
+                const int xs[4] = {x4.x, x4.y, x4.z, x4.w};   // padding is above every id
+#pragma unroll
+                for (int z = 0; z < 4; z++) {
+                    int lo = 0, hi = d - 1;
+                    while (lo < hi) {
+                        const int mid = (lo + hi) >> 1;
+                        if ((small ? sl[mid] : adj[b + mid]) < xs[z]) lo = mid + 1; else hi = mid;
+                    }
+                    c += (small ? sl[lo] : adj[b + lo]) == xs[z] ? 1 : 0;
                 }
-                c += (d > 0 && adj[b + lo] == x) ? 1 : 0;
             }
         }
         c = gpm_warp_sum(c);
         if (lane == 0) tri[v] = (float)c;
+        __syncwarp();
     }
 }
 
-// Core numbers by peeling (the k-core decomposition): at level c every
-// remaining vertex whose remaining degree is <= c gets core number c and is
-// removed, which lowers its remaining neighbours' degrees; a level is
-// repeated until it removes nothing, then c moves to the smallest remaining
-// degree.  One pass of one level: flags[0] = 1 if it removed a vertex,
-// flags[1] = the smallest remaining degree among the vertices it kept.
-__global__ void k_core_init(const int32_t* __restrict__ deg, int32_t n, int32_t* __restrict__ rem,
-                            int32_t* __restrict__ core) {
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-        rem[v] = deg[v];
+// Core numbers by peeling (the k-core decomposition), in one cooperative
+// launch: at level c every remaining vertex whose remaining degree is <= c gets
+// core number c and is removed, which lowers its remaining neighbours' degrees.
+// The vertices that fall to c that way (each noticed by the decrement that
+// takes it from c + 1 to c) form the next round of the level; when a round is
+// empty, a scan of all vertices finds the next level, the smallest remaining
+// degree, and its first round.  Rounds are separated by grid barriers.
+//
+// Bound: the barriers, about one per round and level.  Up to CORE_CLUSTER_N
+// vertices the launch is one cluster of eight blocks, whose barrier is a
+// hardware one; above, one block per SM (the scans of a level need the threads).
+// One launch per pass over all vertices, with the host reading a flag in
+// between, took 55 us a pass: 10.2 ms on rmat14 (185 passes).
+constexpr int CORE_THREADS = 512;
+constexpr int CORE_CLUSTER = 8;
+constexpr int CORE_CLUSTER_N = 1 << 17;
+
+struct CoreState {
+    int n_queue[3];      // sizes of the rounds: current, next, and the one being zeroed
+    int min_left[2];     // smallest remaining degree found by a scan (two in turn)
+};
+
+template <bool CLUSTER>
+__device__ __forceinline__ void core_sync() {
+    if constexpr (CLUSTER) cooperative_groups::this_cluster().sync();
+    else cooperative_groups::this_grid().sync();
+}
+
+template <bool CLUSTER>
+__global__ void __launch_bounds__(CORE_THREADS) k_core(const int32_t* __restrict__ indptr,
+                                                       const int32_t* __restrict__ indices, int32_t n,
+                                                       int32_t* rem, int32_t* core, int32_t* queue0, int32_t* queue1,
+                                                       CoreState* st) {
+    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+    for (long long v = tid; v < n; v += nt) {
+        rem[v] = indptr[v + 1] - indptr[v];
         core[v] = -1;
     }
-}
-
-__global__ void k_core_peel(const int32_t* __restrict__ indptr, const int32_t* __restrict__ indices, int32_t n,
-                            int32_t c, int32_t* __restrict__ rem, int32_t* __restrict__ core, int* __restrict__ flags) {
-    int removed = 0, keep_min = INT32_MAX;
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-        if (core[v] >= 0) continue;
-        const int r = atomicAdd(&rem[v], 0);
-        if (r <= c) {
-            core[v] = c;
-            removed = 1;
-            for (int t = indptr[v]; t < indptr[v + 1]; t++) {
-                const int u = indices[t];
-                if (atomicAdd(&core[u], 0) < 0) atomicSub(&rem[u], 1);
+    if (tid == 0) {
+        st->n_queue[0] = st->n_queue[1] = st->n_queue[2] = 0;
+        st->min_left[0] = st->min_left[1] = INT32_MAX;
+    }
+    core_sync<CLUSTER>();
+    int c = 0, round = 0, scan = 0;
+    for (;;) {
+        // the vertices of level c, and the smallest degree above it
+        int least = INT32_MAX;
+        for (long long v = tid; v < n; v += nt) {
+            if (core[v] >= 0) continue;
+            const int r = rem[v];
+            if (r <= c) {
+                core[v] = c;
+                (round & 1 ? queue1 : queue0)[atomicAdd(&st->n_queue[round % 3], 1)] = (int32_t)v;
+            } else {
+                least = min(least, r);
             }
-        } else {
-            keep_min = min(keep_min, r);
         }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        removed |= __shfl_xor_sync(GPM_FULL_MASK, removed, o);
-        keep_min = min(keep_min, __shfl_xor_sync(GPM_FULL_MASK, keep_min, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (removed) atomicOr(&flags[0], 1);
-        if (keep_min != INT32_MAX) atomicMin(&flags[1], keep_min);
+        least = (int)__reduce_min_sync(GPM_FULL_MASK, (unsigned)least);
+        if ((threadIdx.x & 31) == 0 && least != INT32_MAX) atomicMin(&st->min_left[scan & 1], least);
+        core_sync<CLUSTER>();
+        const int left = *(volatile int*)&st->min_left[scan & 1];
+        const bool none = *(volatile int*)&st->n_queue[round % 3] == 0;
+        if (tid == 0) st->min_left[(scan + 1) & 1] = INT32_MAX;
+        scan++;
+        for (;;) {
+            const int m = *(volatile int*)&st->n_queue[round % 3];
+            if (!m) break;
+            const int32_t* q = round & 1 ? queue1 : queue0;
+            int32_t* next = round & 1 ? queue0 : queue1;
+            // eight lanes per removed vertex
+            for (long long i = tid >> 3; i < m; i += nt >> 3) {
+                const int v = __ldcg(q + i);
+                for (int t = indptr[v] + (int)(tid & 7), e = indptr[v + 1]; t < e; t += 8) {
+                    const int u = indices[t];
+                    if (*(volatile int*)&core[u] >= 0) continue;
+                    if (atomicSub(&rem[u], 1) == c + 1) {
+                        *(volatile int*)&core[u] = c;
+                        next[atomicAdd(&st->n_queue[(round + 1) % 3], 1)] = u;
+                    }
+                }
+            }
+            if (tid == 0) st->n_queue[(round + 2) % 3] = 0;
+            core_sync<CLUSTER>();
+            round++;
+        }
+        if (left == INT32_MAX) break;    // every vertex had level <= c
+        // (the rounds of level c can have brought vertices down to c + 1)
+        c = none ? left : c + 1;
+        core_sync<CLUSTER>();
     }
 }
 
@@ -118,13 +187,20 @@ __global__ void k_features(const int32_t* __restrict__ indptr, const int32_t* __
         const int b = indptr[v], e = indptr[v + 1];
         double s_all = 0, s_up = 0;
         int c_up = 0;
-        for (int t = b + lane; t < e; t += 32) {
-            const int u = indices[t];
-            const int du = deg[u];
-            s_all += du;
-            if (u > v) {
-                s_up += du;
-                c_up++;
+        // four entries per lane in flight: a hub's list is the kernel's time
+        for (int t = b + lane; t < e; t += 128) {
+            int us[4], ds[4];
+#pragma unroll
+            for (int z = 0; z < 4; z++) us[z] = t + 32 * z < e ? indices[t + 32 * z] : -1;
+#pragma unroll
+            for (int z = 0; z < 4; z++) ds[z] = us[z] >= 0 ? deg[us[z]] : 0;
+#pragma unroll
+            for (int z = 0; z < 4; z++) {
+                s_all += ds[z];
+                if (us[z] > v) {
+                    s_up += ds[z];
+                    c_up++;
+                }
             }
         }
         for (int o = 16; o > 0; o >>= 1) {
@@ -151,30 +227,30 @@ static int blocks_for(int64_t items_x32, int threads, int sms) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)sms * 32));
 }
 
-// core numbers of every vertex into d_core (host-driven peeling passes)
+// core numbers of every vertex into d_core
 static void core_numbers(gpm_graph* g, int32_t* d_core, DevBuf& tmp) {
-    cudaStream_t s = g->stream;
-    const int32_t n = g->n;
-    tmp.ensure(sizeof(int32_t) * ((size_t)n + 8));
+    int32_t n = g->n;
+    tmp.ensure(sizeof(int32_t) * 3 * (size_t)n + sizeof(CoreState));
     int32_t* rem = tmp.as<int32_t>();
-    int* flags = reinterpret_cast<int*>(rem + n);
-    const int blocks = blocks_for((int64_t)n, 256, g->num_sms);
-    k_core_init<<<blocks, 256, 0, s>>>(g->degree.as<int32_t>(), n, rem, d_core);
-    GPM_CUDA(cudaGetLastError());
-    int c = 0;
-    for (long long pass = 0;; pass++) {
-        if (pass > 4ll * n + 16) fail(GPM_ECUDA, "core decomposition did not converge");
-        const int init[2] = {0, INT32_MAX};
-        GPM_CUDA(cudaMemcpyAsync(flags, init, sizeof(init), cudaMemcpyHostToDevice, s));
-        k_core_peel<<<blocks, 256, 0, s>>>(g->indptr.as<int32_t>(), g->indices.as<int32_t>(), n, c, rem, d_core,
-                                           flags);
-        GPM_CUDA(cudaGetLastError());
-        int h[2];
-        GPM_CUDA(cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, s));
-        GPM_CUDA(cudaStreamSynchronize(s));
-        if (h[0]) continue;              // level c removed something: run it again
-        if (h[1] == INT32_MAX) break;    // nothing left
-        c = std::max(c + 1, h[1]);
+    int32_t *q0 = rem + n, *q1 = q0 + n;
+    CoreState* st = reinterpret_cast<CoreState*>(q1 + n);
+    const int32_t *indptr = g->indptr.as<int32_t>(), *indices = g->indices.as<int32_t>();
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.blockDim = dim3(CORE_THREADS);
+    cfg.stream = g->stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (n <= CORE_CLUSTER_N) {
+        cfg.gridDim = dim3(CORE_CLUSTER);
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim = {CORE_CLUSTER, 1, 1};
+        GPM_CUDA(cudaLaunchKernelEx(&cfg, k_core<true>, indptr, indices, n, rem, d_core, q0, q1, st));
+    } else {
+        cfg.gridDim = dim3(g->num_sms);
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        GPM_CUDA(cudaLaunchKernelEx(&cfg, k_core<false>, indptr, indices, n, rem, d_core, q0, q1, st));
     }
 }
 
@@ -186,7 +262,7 @@ void root_features(gpm_graph* g, int k, float* d_out) {
     core.ensure(sizeof(int32_t) * std::max(g->n, 1));
     if (g->n > 0) {
         core_numbers(g, core.as<int32_t>(), tmp);
-        k_tri_root<<<blocks_for((int64_t)g->n * 32, 256, g->num_sms), 256, 0, s>>>(
+        k_tri_root<<<blocks_for((int64_t)g->n * 32, TRI_THREADS, g->num_sms), TRI_THREADS, 0, s>>>(
             g->dag_off.as<int32_t>(), g->dag_adj.as<int32_t>(), g->dag_outdeg.as<int32_t>(), g->n, tri.as<float>());
         k_features<<<blocks_for((int64_t)g->n * 32, 256, g->num_sms), 256, 0, s>>>(
             g->indptr.as<int32_t>(), g->indices.as<int32_t>(), g->degree.as<int32_t>(), g->dag_outdeg.as<int32_t>(),
