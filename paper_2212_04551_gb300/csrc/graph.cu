@@ -66,41 +66,46 @@ void DevBuf::ensure(size_t need) {
 
 // --------------------------------------------------------------- kernels
 
-// Warp per vertex: ids in range, no self-loop, strictly ascending, and the
-// reverse edge present (binary search of v in N(x)).
+// Ids in range, no self-loop, strictly ascending, and the reverse edge present
+// (binary search of v in N(x)).  Thread per adjacency entry, whose vertex v it
+// finds in indptr (a warp per vertex left the whole grid waiting for the
+// searches of one hub: 423 us on rmat16); needs a monotone indptr, which
+// k_indptr_monotone has flagged otherwise.
 __global__ void k_validate(const int32_t* __restrict__ indptr, const int32_t* __restrict__ indices,
                            int32_t n, int64_t nnz, int* __restrict__ bad) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t v = warp; v < n; v += nwarps) {
-        const int64_t s = indptr[v], e = indptr[v + 1];
-        if (s < 0 || e < s || e > nnz) {
-            if (lane == 0) atomicOr(bad, 1);
-            continue;
+    int b = 0;
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t x = indices[p];
+        // the last vertex whose list begins at or before p
+        int32_t lo = 0, hi = n - 1;
+        while (lo < hi) {
+            const int32_t mid = (int32_t)(((int64_t)lo + hi + 1) >> 1);
+            if (indptr[mid] <= p) lo = mid; else hi = mid - 1;
         }
-        for (int64_t p = s + lane; p < e; p += 32) {
-            const int32_t x = indices[p];
-            int b = 0;
-            if (x < 0 || x >= n) b |= 2;
-            else {
-                if (x == v) b |= 4;
-                if (p > s && indices[p - 1] >= x) b |= 8;
-                int64_t lo = indptr[x], hi = indptr[x + 1] - 1;
-                bool found = false;
-                if (lo >= 0 && hi < nnz) {
-                    while (lo <= hi) {
-                        const int64_t mid = (lo + hi) >> 1;
-                        const int32_t y = indices[mid];
-                        if (y == (int32_t)v) { found = true; break; }
-                        if (y < (int32_t)v) lo = mid + 1; else hi = mid - 1;
-                    }
+        const int32_t v = lo;
+        const int64_t s = indptr[v];
+        if (s < 0 || p >= indptr[v + 1]) {
+            b |= 1;
+        } else if (x < 0 || x >= n) {
+            b |= 2;
+        } else {
+            if (x == v) b |= 4;
+            if (p > s && indices[p - 1] >= x) b |= 8;
+            int64_t l = indptr[x], h = (int64_t)indptr[x + 1] - 1;
+            bool found = false;
+            if (l >= 0 && h < nnz) {
+                while (l <= h) {
+                    const int64_t mid = (l + h) >> 1;
+                    const int32_t y = indices[mid];
+                    if (y == v) { found = true; break; }
+                    if (y < v) l = mid + 1; else h = mid - 1;
                 }
-                if (!found) b |= 16;
             }
-            if (b) atomicOr(bad, b);
+            if (!found) b |= 16;
         }
     }
+    b = (int)__reduce_or_sync(GPM_FULL_MASK, (unsigned)b);
+    if (b && (threadIdx.x & 31) == 0) atomicOr(bad, b);
 }
 
 __global__ void k_indptr_monotone(const int32_t* __restrict__ indptr, int32_t n, int* __restrict__ bad) {
@@ -131,20 +136,30 @@ __global__ void k_outdeg(const int32_t* __restrict__ indptr, const int32_t* __re
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    int most = 0;
     for (int64_t v = warp; v < n; v += nwarps) {
         const int32_t dv = deg[v];
         int c = 0;
-        for (int64_t p = indptr[v] + lane; p < indptr[v + 1]; p += 32) {
-            const int32_t x = indices[p];
-            c += dag_before(dv, (int32_t)v, deg[x], x) ? 1 : 0;
+        // four entries per lane in flight: a hub's list is the kernel's time
+        const int64_t e = indptr[v + 1];
+        for (int64_t p = indptr[v] + lane; p < e; p += 128) {
+            int32_t xs[4], dx[4];
+#pragma unroll
+            for (int z = 0; z < 4; z++) xs[z] = p + 32 * z < e ? indices[p + 32 * z] : -1;
+#pragma unroll
+            for (int z = 0; z < 4; z++) dx[z] = xs[z] >= 0 ? deg[xs[z]] : -1;
+#pragma unroll
+            for (int z = 0; z < 4; z++) c += xs[z] >= 0 && dag_before(dv, (int32_t)v, dx[z], xs[z]) ? 1 : 0;
         }
         c = gpm_warp_sum(c);
         if (lane == 0) {
             outdeg[v] = c;
             padded[v] = (c + 3) & ~3;
-            atomicMax(maxout, c);
         }
+        most = max(most, c);
     }
+    // (one add per vertex on the same word took most of the kernel's time)
+    if (lane == 0 && most) atomicMax(maxout, most);
 }
 
 __global__ void k_dag_fill(const int32_t* __restrict__ indptr, const int32_t* __restrict__ indices,
@@ -157,17 +172,20 @@ __global__ void k_dag_fill(const int32_t* __restrict__ indptr, const int32_t* __
         const int32_t dv = deg[v];
         int64_t base = off[v];
         const int64_t end = off[v + 1];
-        for (int64_t p0 = indptr[v]; p0 < indptr[v + 1]; p0 += 32) {
-            const int64_t p = p0 + lane;
-            bool keep = false;
-            int32_t x = 0;
-            if (p < indptr[v + 1]) {
-                x = indices[p];
-                keep = dag_before(dv, (int32_t)v, deg[x], x);
+        const int64_t pe = indptr[v + 1];
+        for (int64_t p = indptr[v] + lane; p - lane < pe; p += 128) {
+            int32_t xs[4], dx[4];
+#pragma unroll
+            for (int z = 0; z < 4; z++) xs[z] = p + 32 * z < pe ? indices[p + 32 * z] : -1;
+#pragma unroll
+            for (int z = 0; z < 4; z++) dx[z] = xs[z] >= 0 ? deg[xs[z]] : -1;
+#pragma unroll
+            for (int z = 0; z < 4; z++) {
+                const bool keep = xs[z] >= 0 && dag_before(dv, (int32_t)v, dx[z], xs[z]);
+                const unsigned bal = __ballot_sync(GPM_FULL_MASK, keep);
+                if (keep) adj[base + __popc(bal & gpm_lanemask_lt())] = xs[z];
+                base += __popc(bal);
             }
-            const unsigned bal = __ballot_sync(GPM_FULL_MASK, keep);
-            if (keep) adj[base + __popc(bal & gpm_lanemask_lt())] = x;
-            base += __popc(bal);
         }
         for (int64_t p = base + lane; p < end; p += 32) adj[p] = INT32_MAX;
     }
@@ -264,15 +282,30 @@ void exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, int64_t* tot
 
 __global__ void k_key_hist(const int32_t* __restrict__ key, int32_t n, int32_t maxkey,
                            int32_t* __restrict__ hist) {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&hist[maxkey - min(key[v], maxkey)], 1);
+    // one add per distinct key of a warp: most vertices share a few small keys
+    const int lane = threadIdx.x & 31;
+    for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); v0 < n;
+         v0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t v = v0 + lane;
+        const int bin = v < n ? maxkey - min(key[v], maxkey) : -1;
+        const unsigned same = __match_any_sync(GPM_FULL_MASK, bin);
+        if (bin >= 0 && lane == __ffs(same) - 1) atomicAdd(&hist[bin], __popc(same));
+    }
 }
 
 __global__ void k_key_scatter(const int32_t* __restrict__ key, int32_t n, int32_t maxkey,
                               int32_t* __restrict__ cursor, int32_t* __restrict__ order) {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        const int pos = atomicAdd(&cursor[maxkey - min(key[v], maxkey)], 1);
-        order[pos] = (int32_t)v;
+    const int lane = threadIdx.x & 31;
+    for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); v0 < n;
+         v0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t v = v0 + lane;
+        const int bin = v < n ? maxkey - min(key[v], maxkey) : -1;
+        const unsigned same = __match_any_sync(GPM_FULL_MASK, bin);
+        const int first = __ffs(same) - 1;
+        int pos = 0;
+        if (bin >= 0 && lane == first) pos = atomicAdd(&cursor[bin], __popc(same));
+        pos = __shfl_sync(GPM_FULL_MASK, pos, first) + __popc(same & gpm_lanemask_lt());
+        if (bin >= 0) order[pos] = (int32_t)v;
     }
 }
 
@@ -457,7 +490,7 @@ gpm_graph* create_graph(const int32_t* indptr, const int32_t* indices, int32_t n
         g->max_deg = hb[1];
         if (!(flags & GPM_SKIP_VALIDATE) && n > 0 && last > 0) {
             GPM_CUDA(cudaMemsetAsync(flag.ptr, 0, sizeof(int), s));
-            k_validate<<<grid_for((int64_t)n * 32, 256, g->num_sms), 256, 0, s>>>(
+            k_validate<<<grid_for(last, 256, g->num_sms), 256, 0, s>>>(
                 g->indptr.as<int32_t>(), g->indices.as<int32_t>(), n, last, bad);
             GPM_CUDA(cudaGetLastError());
             int v = 0;
