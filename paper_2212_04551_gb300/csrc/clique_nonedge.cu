@@ -33,8 +33,8 @@
 // are therefore not unrolled: with the compiler's unrolling the heavy kernel
 // was 401 KB of code instead of 113 KB, and 81 ms instead of 34.  The light
 // launch is bound by the latency of its chain of dependent loads per root.
-// Measured, whole call on that graph: k = 4..7 1,378 -> 36 ms, k = 4 8.0 ->
-// 4.0 ms; block-model graph of 2,000 vertices, k = 6..12: 20.9 -> 0.6 ms.
+// Measured, whole call on that graph: k = 4..7 1,378 -> 35 ms, k = 4 8.0 ->
+// 2.8 ms; block-model graph of 2,000 vertices, k = 6..12: 20.9 -> 0.6 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -193,7 +193,6 @@ __global__ void __launch_bounds__(NE_LIGHT_WARPS * 32) k_clique_ne_light(NeLaunc
                 __syncwarp();
             }
         }
-        ne_fold(p.ne, c, lane);
         units += (unsigned)nr;
     }
     busy = gpm_globaltimer() - t0;
@@ -205,7 +204,8 @@ __global__ void __launch_bounds__(NE_LIGHT_WARPS * 32) k_clique_ne_light(NeLaunc
 // shared words of one warp: a candidate bitmap per level, the member lists
 // (16-bit positions; of the current set, and of a wide set with the non-edges
 // of each), the re-indexed rows and their level stack
-__host__ __device__ inline int ne_warp_words(int maxd, int w) {
+__host__ __device__ inline int ne_warp_words(int maxd, int w, bool deep) {
+    if (!deep) return 3 * w + ((maxd + 3) & ~3) / 2;
     return NE_LEVELS * w + 3 * ((maxd + 3) & ~3) / 2 + 32 * NE_W * NE_W + NE_W * NE_LEVELS + NE_SCRATCH;
 }
 
@@ -413,7 +413,11 @@ __device__ __forceinline__ void ne_child(const NeLaunch& p, NeCount& c, const Ne
     }
 }
 
-__global__ void __launch_bounds__(NE_WARPS * 32) k_clique_ne_heavy(NeLaunch p) {
+// DEEP: three sizes or more to go below a child (k >= 5); without, neither the
+// re-indexed rows nor their registers are there (48 instead of 96), and twice
+// the warps are resident: k = 4 on the Chung-Lu graph 4.0 -> 2.8 ms.
+template <bool DEEP>
+__global__ void __launch_bounds__(NE_WARPS * 32, DEEP ? 5 : 10) k_clique_ne_heavy(NeLaunch p) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ unsigned long long s_pos;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -425,12 +429,18 @@ __global__ void __launch_bounds__(NE_WARPS * 32) k_clique_ne_heavy(NeLaunch p) {
     uint32_t* mine = smem + ne_block_words(p.maxd, p.ws) + wib * p.warp_words;
     NeWarp k;
     k.cand = mine;
-    k.Hs = k.cand + NE_LEVELS * p.w;
-    k.stk = k.Hs + 32 * NE_W * NE_W;
-    k.scratch = k.stk + NE_W * NE_LEVELS;
-    k.mem = reinterpret_cast<uint16_t*>(k.scratch + NE_SCRATCH);
-    k.wide = k.mem + dpad;
-    k.we = k.wide + dpad;
+    if (DEEP) {
+        k.Hs = k.cand + NE_LEVELS * p.w;
+        k.stk = k.Hs + 32 * NE_W * NE_W;
+        k.scratch = k.stk + NE_W * NE_LEVELS;
+        k.mem = reinterpret_cast<uint16_t*>(k.scratch + NE_SCRATCH);
+        k.wide = k.mem + dpad;
+        k.we = k.wide + dpad;
+    } else {
+        k.Hs = k.stk = k.scratch = nullptr;
+        k.mem = reinterpret_cast<uint16_t*>(k.cand + 3 * p.w);
+        k.wide = k.we = nullptr;
+    }
     const unsigned long long n_own = (unsigned long long)(p.last - p.first);
     const unsigned long long n_offers = n_own + (unsigned long long)p.n_help * p.rounds;
     NeCount c;
@@ -539,11 +549,16 @@ __global__ void __launch_bounds__(NE_WARPS * 32) k_clique_ne_heavy(NeLaunch p) {
                     C[lane] = rows[q * p.ws + lane] & after;
                 }
                 __syncwarp();
-                ne_child(p, c, k, rows, w, lane);
+                if (DEEP) {
+                    ne_child(p, c, k, rows, w, lane);
+                } else {
+                    int m, a;
+                    ne_node(p, c, k, rows, w, C, 2, m, a, lane);   // two sizes to go at most: counted
+                }
                 __syncwarp();
             }
-            ne_fold(p.ne, c, lane);
         }
+        if (DEEP) ne_fold(p.ne, c, lane);
         if (threadIdx.x == 0) units++;
         busy += gpm_globaltimer() - t_unit;
     }
@@ -618,17 +633,20 @@ int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* 
         p.maxd = std::min(g->max_outdeg, NE_BINOM_N);
         p.w = (p.maxd + 31) / 32;
         p.ws = p.w | 1;
-        p.warp_words = ne_warp_words(p.maxd, p.w);
+        const bool deep = k_hi >= 5;
+        const void* heavy = deep ? (const void*)k_clique_ne_heavy<true> : (const void*)k_clique_ne_heavy<false>;
+        p.warp_words = ne_warp_words(p.maxd, p.w, deep);
         p.n_help = std::max(0ll, roots_at_least(g, NE_HELP_D + 1) - above);
         p.rounds = k_hi >= 6 ? NE_HELP_ROUNDS : 0;
         p.grab = k_hi >= 6 ? 2 : 16;
         p.ticket = tickets;
         p.next_child = reinterpret_cast<unsigned int*>(tickets + 32);
         const size_t smem = 4 * ((size_t)ne_block_words(p.maxd, p.ws) + (size_t)NE_WARPS * p.warp_words);
-        GPM_CUDA(cudaFuncSetAttribute(k_clique_ne_heavy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        Grid gr = plan_grid(g, (const void*)k_clique_ne_heavy, NE_WARPS, smem);
+        GPM_CUDA(cudaFuncSetAttribute(heavy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        Grid gr = plan_grid(g, heavy, NE_WARPS, smem);
         gr.blocks = (int)std::min<long long>(gr.blocks, n_big + p.n_help * p.rounds);
-        k_clique_ne_heavy<<<gr.blocks, NE_WARPS * 32, smem, s>>>(p);
+        if (deep) k_clique_ne_heavy<true><<<gr.blocks, NE_WARPS * 32, smem, s>>>(p);
+        else k_clique_ne_heavy<false><<<gr.blocks, NE_WARPS * 32, smem, s>>>(p);
         GPM_CUDA(cudaGetLastError());
         *grid = gr;
         launches++;
