@@ -311,98 +311,170 @@ __global__ void __launch_bounds__(256) k_mlp_forward(const uint16_t* __restrict_
     }
 }
 
-// Gradients of mean_i (y_i - t_i)^2 over a minibatch of n samples.  A block
-// handles 64 samples at a time: one thread per sample computes the forward
-// and the per-sample deltas into shared memory, then the block forms the
-// weight gradients as sums over its samples and adds them to grad (FP32
-// atomics).  grad and loss must be zero on entry.
-constexpr int BW_TILE = 64;
-__global__ void __launch_bounds__(BW_TILE) k_mlp_backward(const uint16_t* __restrict__ w, const float* __restrict__ x,
-                                                          const float* __restrict__ t, long long n,
-                                                          float* __restrict__ grad, float* __restrict__ loss) {
+// Gradients of mean_i (y_i - t_i)^2 over a minibatch of n samples.  A block of
+// 256 threads takes BW_TILE samples at a time; every product of the pass is a
+// small matrix product over shared memory with a register tile per thread:
+//
+//   z1 = x W1' + b1, z2 = relu(z1) W2' + b2, D1 = (D2 W2) .* [z1 > 0]   tile x 64, 4 x 2 per thread
+//   dW2 += D2' relu(z1)   64 x 64, 4 x 4 per thread, kept over the block's tiles
+//   dW1 += D1' x          64 x 8, 2 per thread
+//
+// and the block adds its sums to grad once (FP32 atomics).  grad and loss must
+// be zero on entry.  Bound: the latency of the phases of one tile (a minibatch
+// of 4,096 is one tile per block) and the atomics.  With one thread per sample
+// and rows of dW2 per thread, 64 threads per block, it took 65 us at n = 4,096.
+constexpr int BW_TILE = 32;
+constexpr int BW_THREADS = 256;
+constexpr int BW_S = MLP_H + 1;                      // row stride of the 64-wide arrays
+constexpr int BW_SMEM = MLP_NPARAM + 3 + BW_TILE * MLP_IN + 4 * BW_TILE * BW_S + BW_TILE;
+__global__ void __launch_bounds__(BW_THREADS) k_mlp_backward(const uint16_t* __restrict__ w,
+                                                             const float* __restrict__ x, const float* __restrict__ t,
+                                                             long long n, float* __restrict__ grad,
+                                                             float* __restrict__ loss) {
     extern __shared__ float sh[];
     float* W = sh;                                   // MLP_NPARAM
     float* X = W + MLP_NPARAM + 3;                   // BW_TILE x 8
-    float* H1 = X + BW_TILE * MLP_IN;                // BW_TILE x 65
-    float* H2 = H1 + BW_TILE * (MLP_H + 1);
-    float* D2 = H2 + BW_TILE * (MLP_H + 1);          // dL/dz2
-    float* D1 = D2 + BW_TILE * (MLP_H + 1);          // dL/dz1
-    float* DY = D1 + BW_TILE * (MLP_H + 1);          // dL/dy
+    float* H1 = X + BW_TILE * MLP_IN;                // relu(z1)
+    float* H2 = H1 + BW_TILE * BW_S;                 // relu(z2)
+    float* D2 = H2 + BW_TILE * BW_S;                 // dL/dz2
+    float* D1 = D2 + BW_TILE * BW_S;                 // dL/dz1
+    float* DY = D1 + BW_TILE * BW_S;                 // dL/dy
     load_weights(w, W);
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const float inv_n = 1.0f / (float)n;
-    float lsum = 0.f;
-    // per-thread accumulators for the entries this thread owns
-    float gW2[MLP_H];                                // row tid of dW2 (64 entries)
-    float gW1[MLP_IN];                               // row tid of dW1
-    float gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f;
+    // tile x 64 products: samples s0 .. s0 + 3, neurons j0 and j0 + 32
+    const int s0 = 4 * wid, j0 = lane;
+    // 64 x 64 gradient: rows r0 .. r0 + 3, columns q0, q0 + 16, q0 + 32, q0 + 48
+    const int r0 = 4 * (tid >> 4), q0 = tid & 15;
+    float gW2[4][4], gW1[2] = {0.f, 0.f}, gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f, lsum = 0.f;
 #pragma unroll
-    for (int q = 0; q < MLP_H; q++) gW2[q] = 0.f;
+    for (int i = 0; i < 4; i++)
 #pragma unroll
-    for (int q = 0; q < MLP_IN; q++) gW1[q] = 0.f;
+        for (int q = 0; q < 4; q++) gW2[i][q] = 0.f;
 
     for (long long base = (long long)blockIdx.x * BW_TILE; base < n; base += (long long)gridDim.x * BW_TILE) {
-        const long long i = base + tid;
-        const bool act = i < n;
-        float xi[MLP_IN];
+        for (int i = tid; i < BW_TILE * MLP_IN; i += BW_THREADS)
+            X[i] = base + i / MLP_IN < n ? x[base * MLP_IN + i] : 0.f;
+        __syncthreads();
+        // z1
 #pragma unroll
-        for (int q = 0; q < MLP_IN; q++) {
-            xi[q] = act ? x[i * MLP_IN + q] : 0.f;
-            X[tid * MLP_IN + q] = xi[q];
-        }
-        for (int j = 0; j < MLP_H; j++) {
-            float s = W[OFF_B1 + j];
+        for (int jj = 0; jj < 2; jj++) {
+            const int j = j0 + 32 * jj;
+            float wj[MLP_IN];
 #pragma unroll
-            for (int q = 0; q < MLP_IN; q++) s = fmaf(W[OFF_W1 + j * MLP_IN + q], xi[q], s);
-            H1[tid * (MLP_H + 1) + j] = s;           // z1 for now
+            for (int q = 0; q < MLP_IN; q++) wj[q] = W[OFF_W1 + j * MLP_IN + q];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                float s = W[OFF_B1 + j];
+#pragma unroll
+                for (int q = 0; q < MLP_IN; q++) s = fmaf(wj[q], X[(s0 + i) * MLP_IN + q], s);
+                H1[(s0 + i) * BW_S + j] = fmaxf(s, 0.f);
+            }
         }
-        float yv = W[OFF_B3];
-        for (int j = 0; j < MLP_H; j++) {
-            float s = W[OFF_B2 + j];
-            for (int q = 0; q < MLP_H; q++) s = fmaf(W[OFF_W2 + j * MLP_H + q], fmaxf(H1[tid * (MLP_H + 1) + q], 0.f), s);
-            H2[tid * (MLP_H + 1) + j] = s;           // z2 for now
-            yv = fmaf(W[OFF_W3 + j], fmaxf(s, 0.f), yv);
+        __syncwarp();                                // (a warp's samples are its own until D1 is there)
+        // z2
+        float z[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            z[i][0] = W[OFF_B2 + j0];
+            z[i][1] = W[OFF_B2 + j0 + 32];
         }
-        const float diff = act ? (yv - t[i]) : 0.f;
-        lsum += diff * diff;
-        const float dy = 2.f * diff * inv_n;
-        DY[tid] = dy;
-        for (int j = 0; j < MLP_H; j++) {
-            const float z2 = H2[tid * (MLP_H + 1) + j];
-            D2[tid * (MLP_H + 1) + j] = z2 > 0.f ? dy * W[OFF_W3 + j] : 0.f;
-        }
+#pragma unroll 8
         for (int q = 0; q < MLP_H; q++) {
-            float s = 0.f;
-            for (int j = 0; j < MLP_H; j++) s = fmaf(D2[tid * (MLP_H + 1) + j], W[OFF_W2 + j * MLP_H + q], s);
-            const float z1 = H1[tid * (MLP_H + 1) + q];
-            D1[tid * (MLP_H + 1) + q] = z1 > 0.f ? s : 0.f;
+            const float w0 = W[OFF_W2 + j0 * MLP_H + ((q + j0) & 63)], w1 = W[OFF_W2 + (j0 + 32) * MLP_H + ((q + j0) & 63)];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const float h = H1[(s0 + i) * BW_S + ((q + j0) & 63)];
+                z[i][0] = fmaf(w0, h, z[i][0]);
+                z[i][1] = fmaf(w1, h, z[i][1]);
+            }
+        }
+        // y, dy, D2
+        const float v0 = W[OFF_W3 + j0], v1 = W[OFF_W3 + j0 + 32];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const float h0 = fmaxf(z[i][0], 0.f), h1 = fmaxf(z[i][1], 0.f);
+            const float y = gpm_warp_sum(fmaf(v0, h0, v1 * h1)) + W[OFF_B3];
+            const long long g = base + s0 + i;
+            const float diff = g < n ? y - t[g] : 0.f;
+            const float dy = 2.f * diff * inv_n;
+            if (lane == 0) {
+                DY[s0 + i] = dy;
+                lsum += diff * diff;
+            }
+            H2[(s0 + i) * BW_S + j0] = h0;
+            H2[(s0 + i) * BW_S + j0 + 32] = h1;
+            D2[(s0 + i) * BW_S + j0] = z[i][0] > 0.f ? dy * v0 : 0.f;
+            D2[(s0 + i) * BW_S + j0 + 32] = z[i][1] > 0.f ? dy * v1 : 0.f;
+        }
+        __syncwarp();
+        // D1
+        float d[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; i++) d[i][0] = d[i][1] = 0.f;
+#pragma unroll 8
+        for (int q = 0; q < MLP_H; q++) {
+            const float w0 = W[OFF_W2 + q * MLP_H + j0], w1 = W[OFF_W2 + q * MLP_H + j0 + 32];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const float e = D2[(s0 + i) * BW_S + q];
+                d[i][0] = fmaf(e, w0, d[i][0]);
+                d[i][1] = fmaf(e, w1, d[i][1]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            D1[(s0 + i) * BW_S + j0] = H1[(s0 + i) * BW_S + j0] > 0.f ? d[i][0] : 0.f;
+            D1[(s0 + i) * BW_S + j0 + 32] = H1[(s0 + i) * BW_S + j0 + 32] > 0.f ? d[i][1] : 0.f;
         }
         __syncthreads();
-        // thread tid owns row j = tid of dW2, dW1 and entry j of b1, b2, w3
-        const int j = tid;
-        for (int sidx = 0; sidx < BW_TILE; sidx++) {
-            const float d2 = D2[sidx * (MLP_H + 1) + j];
-            const float d1 = D1[sidx * (MLP_H + 1) + j];
+        // dW2
+#pragma unroll 4
+        for (int s = 0; s < BW_TILE; s++) {
+            float e[4], h[4];
 #pragma unroll
-            for (int q = 0; q < MLP_H; q++) gW2[q] = fmaf(d2, fmaxf(H1[sidx * (MLP_H + 1) + q], 0.f), gW2[q]);
+            for (int i = 0; i < 4; i++) e[i] = D2[s * BW_S + r0 + i];
 #pragma unroll
-            for (int q = 0; q < MLP_IN; q++) gW1[q] = fmaf(d1, X[sidx * MLP_IN + q], gW1[q]);
-            gb1 += d1;
-            gb2 += d2;
-            gw3 = fmaf(DY[sidx], fmaxf(H2[sidx * (MLP_H + 1) + j], 0.f), gw3);
-            if (j == 0) gb3 += DY[sidx];
+            for (int q = 0; q < 4; q++) h[q] = H1[s * BW_S + q0 + 16 * q];
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+#pragma unroll
+                for (int q = 0; q < 4; q++) gW2[i][q] = fmaf(e[i], h[q], gW2[i][q]);
+        }
+        // dW1: entries tid and tid + 256 (row j, column q); the vectors: a warp pair each
+        {
+            const int j = tid >> 3, q = tid & 7;
+#pragma unroll 8
+            for (int s = 0; s < BW_TILE; s++) {
+                const float xv = X[s * MLP_IN + q];
+                gW1[0] = fmaf(D1[s * BW_S + j], xv, gW1[0]);
+                gW1[1] = fmaf(D1[s * BW_S + j + 32], xv, gW1[1]);
+            }
+        }
+        const int j = tid & 63, part = tid >> 6;     // 0: b1, 1: b2, 2: w3, 3: b3
+        if (part == 0) {
+            for (int s = 0; s < BW_TILE; s++) gb1 += D1[s * BW_S + j];
+        } else if (part == 1) {
+            for (int s = 0; s < BW_TILE; s++) gb2 += D2[s * BW_S + j];
+        } else if (part == 2) {
+            for (int s = 0; s < BW_TILE; s++) gw3 = fmaf(DY[s], H2[s * BW_S + j], gw3);
+        } else if (j == 0) {
+            for (int s = 0; s < BW_TILE; s++) gb3 += DY[s];
         }
         __syncthreads();
     }
-    const int j = tid;
-    for (int q = 0; q < MLP_H; q++) atomicAdd(&grad[OFF_W2 + j * MLP_H + q], gW2[q]);
-    for (int q = 0; q < MLP_IN; q++) atomicAdd(&grad[OFF_W1 + j * MLP_IN + q], gW1[q]);
-    atomicAdd(&grad[OFF_B1 + j], gb1);
-    atomicAdd(&grad[OFF_B2 + j], gb2);
-    atomicAdd(&grad[OFF_W3 + j], gw3);
-    if (j == 0) atomicAdd(&grad[OFF_B3], gb3);
-    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(GPM_FULL_MASK, lsum, o);
-    if ((tid & 31) == 0) atomicAdd(loss, lsum * inv_n);
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) atomicAdd(&grad[OFF_W2 + (r0 + i) * MLP_H + q0 + 16 * q], gW2[i][q]);
+    atomicAdd(&grad[OFF_W1 + tid], gW1[0]);
+    atomicAdd(&grad[OFF_W1 + tid + 256], gW1[1]);
+    const int j = tid & 63, part = tid >> 6;
+    if (part == 0) atomicAdd(&grad[OFF_B1 + j], gb1);
+    else if (part == 1) atomicAdd(&grad[OFF_B2 + j], gb2);
+    else if (part == 2) atomicAdd(&grad[OFF_W3 + j], gw3);
+    else if (j == 0) atomicAdd(&grad[OFF_B3], gb3);
+    if (lane == 0) atomicAdd(loss, lsum * inv_n);
 }
 
 // Adam (Kingma & Ba 2015), bias-corrected; master weights FP32, BF16 copy out
@@ -441,10 +513,10 @@ void mlp_grad(const uint16_t* w, const float* x, const float* t, int64_t n, floa
     int dev = 0, sms = 0;
     GPM_CUDA(cudaGetDevice(&dev));
     GPM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const size_t smem = sizeof(float) * (MLP_NPARAM + 3 + BW_TILE * MLP_IN + 4 * BW_TILE * (MLP_H + 1) + BW_TILE);
+    const size_t smem = sizeof(float) * BW_SMEM;
     GPM_CUDA(cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const int blocks = (int)std::min<int64_t>((n + BW_TILE - 1) / BW_TILE, (int64_t)sms * 4);
-    k_mlp_backward<<<blocks, BW_TILE, smem, s>>>(w, x, t, n, grad, loss);
+    const int blocks = (int)std::min<int64_t>((n + BW_TILE - 1) / BW_TILE, (int64_t)sms * 2);
+    k_mlp_backward<<<blocks, BW_THREADS, smem, s>>>(w, x, t, n, grad, loss);
     GPM_CUDA(cudaGetLastError());
 }
 
