@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(512, 2) k_motif(MotifParams p) {
 
     bool idle = false;
     unsigned long long polls = 0;
-    unsigned long long scanned = 0;   // adjacency entries scanned by this warp (lane 0)
+    unsigned long long scanned = 0;   // adjacency entries scanned by this warp (lane-private)
     int spin = 0;
     long long last_pending = -1;
     unsigned long long idle_since = 0;
@@ -269,6 +269,7 @@ __global__ void __launch_bounds__(512, 2) k_motif(MotifParams p) {
 
     if (lane == 0 && polls) atomicAdd(&ctl->idle_polls, polls);
     if (lane == 0) atomicAdd(&ctl->busy_ns, busy);
+    scanned = gpm_warp_sum(scanned);
     if (lane == 0 && scanned) atomicAdd(&ctl->word_ops, scanned);
     __syncthreads();
     if (!GCOUNT && !LIST)

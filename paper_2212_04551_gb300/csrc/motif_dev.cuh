@@ -45,6 +45,7 @@ constexpr float MT_ENTRIES = 32.f;
 constexpr float MT_NODE = 512.f;
 constexpr int MT_MIN_LEFT = (int)(4 * MT_MIN_DONATE_WORK / MT_ENTRIES);   // children that always make such a range
 constexpr int MT_AGG_UNROLL = 4;                 // adjacency entries per lane per round (mt_tail_agg)
+constexpr int MT_LONG_LIST = 256;                // lists above this are scanned by the whole warp
 
 // A work unit: the children at positions [lo, hi) of the extension array of
 // the node tr = (sub[0], .., sub[depth-1]) (hi < 0: all of them).  The node's
@@ -414,9 +415,11 @@ __device__ __forceinline__ int mt_above_lane(const int32_t* __restrict__ indices
 //   * exclusive neighbours: counted per class of w during the same scans.
 //
 // One scan of N(w) per child replaces the per-leaf walk over the later
-// entries (quadratic in L).  Children are done 32 at a time, their adjacency
-// lists scanned as one flattened range, so that every lane has an entry
-// whatever the degrees.  During the call mark bit 6 flags the entries not done
+// entries (quadratic in L).  Children are done 32 at a time, eight lanes per
+// adjacency list (as one flattened range every lane had an entry whatever the
+// degrees, but had to find that entry's child: block-model graph of 2,000
+// vertices, per-root 5-motifs 68 against 47 ms, 6-motifs 6.2 against 4.4 s;
+// rmat12, whose lists are short, 84 against 82 ms).  During the call mark bit 6 flags the entries not done
 // yet and bit 5 those of the current 32 (free at this level: tr uses bits
 // 0 .. k-3 and 7): an adjacent entry counts if it is not done, and within the
 // 32 from its smaller endpoint.  The counts are then those of the children
@@ -471,63 +474,50 @@ __device__ __noinline__ void mt_tail_agg(const MotifWalk& a, MtWarp* W, int l, c
         }
         __syncwarp();
         const int len = e - b;
-        int incl = len;
+        scanned += (unsigned)len;
+        // one child's entries q, q + stride, ...: MT_AGG_UNROLL per lane per round,
+        // their loads issued together (the mark loads are random and
+        // latency-bound); returns the lane's exclusive neighbours
+        auto scan = [&](int q, int qe, int stride, int ww, int ss) {
+            unsigned exc = 0;
+            for (; q < qe; q += MT_AGG_UNROLL * stride) {
+                int xs[MT_AGG_UNROLL];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(GPM_FULL_MASK, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const int pre = incl - len;
-        const int total = __shfl_sync(GPM_FULL_MASK, incl, 31);
-        if (lane == 0) scanned += (unsigned)total;
-        // MT_AGG_UNROLL entries per lane per round, their loads issued
-        // together (the mark loads are random and latency-bound)
-        for (int f0 = 0; f0 < total; f0 += 32 * MT_AGG_UNROLL) {
-            int xs[MT_AGG_UNROLL], wts[MT_AGG_UNROLL], sts[MT_AGG_UNROLL];
+                for (int u = 0; u < MT_AGG_UNROLL; u++) xs[u] = q + u * stride < qe ? a.indices[q + u * stride] : -1;
+                unsigned ms[MT_AGG_UNROLL];
 #pragma unroll
-            for (int u = 0; u < MT_AGG_UNROLL; u++) {
-                const int f = f0 + 32 * u + lane;
-                int t = 0;                       // owner: the last lane with pre <= f
+                for (int u = 0; u < MT_AGG_UNROLL; u++) ms[u] = xs[u] >= 0 ? a.mk[xs[u] - a.mbase] : 0x80u;
 #pragma unroll
-                for (int step = 16; step > 0; step >>= 1) {
-                    const int pc = __shfl_sync(GPM_FULL_MASK, pre, t + step);
-                    if (pc <= f) t += step;
-                }
-                wts[u] = __shfl_sync(GPM_FULL_MASK, w, t);
-                sts[u] = __shfl_sync(GPM_FULL_MASK, sw, t);
-                const int bt = __shfl_sync(GPM_FULL_MASK, b, t);
-                const int pt = __shfl_sync(GPM_FULL_MASK, pre, t);
-                xs[u] = f < total ? a.indices[bt + (f - pt)] : -1;
-            }
-            unsigned char ms[MT_AGG_UNROLL];
-#pragma unroll
-            for (int u = 0; u < MT_AGG_UNROLL; u++) ms[u] = xs[u] >= 0 ? a.mk[xs[u] - a.mbase] : (unsigned char)0;
-#pragma unroll
-            for (int u = 0; u < MT_AGG_UNROLL; u++) {
-                bool ex = false;
-                if (xs[u] >= 0) {
+                for (int u = 0; u < MT_AGG_UNROLL; u++) {
                     const unsigned m = ms[u];
-                    if ((m & (lowtr | 0x80u)) == 0) {
-                        ex = true;                   // exclusive neighbour of w
-                    } else if ((m & 0x40u) && (!(m & 0x20u) || xs[u] > wts[u])) {
-                        const int s2 = (int)(m & lowtr);   // adjacent pair of entries (rare)
-                        atomicAdd(&P[min(sts[u], s2) * C + max(sts[u], s2)], 1u);
+                    exc += (m & (lowtr | 0x80u)) == 0 ? 1u : 0u;
+                    if ((m & 0x40u) && (!(m & 0x20u) || xs[u] > ww)) {
+                        const int s2 = (int)(m & lowtr);   // adjacent pair of entries
+                        atomicAdd(&P[min(ss, s2) * C + max(ss, s2)], 1u);
                     }
                 }
-                // exclusive neighbours per child: the lanes of one child are
-                // contiguous, so the first lane of each child's run adds the
-                // run's count (children of one class may share a counter)
-                const unsigned exm = __ballot_sync(GPM_FULL_MASK, ex);
-                const int wprev = __shfl_up_sync(GPM_FULL_MASK, wts[u], 1);
-                const bool head = xs[u] >= 0 && (lane == 0 || wprev != wts[u]);
-                const unsigned heads = __ballot_sync(GPM_FULL_MASK, head);
-                if (head) {
-                    const unsigned later = heads & ~((2u << lane) - 1u);   // heads above this lane
-                    const unsigned run = (later ? ((1u << (__ffs(later) - 1)) - 1u) : 0xffffffffu) & ~((1u << lane) - 1u);
-                    const unsigned cnt = (unsigned)__popc(exm & run);
-                    if (cnt) atomicAdd(&E[sts[u]], cnt);
-                }
             }
+            return exc;
+        };
+        // long lists by the whole warp, one after the other; the others by eight
+        // lanes each, four at a time
+        const unsigned longs = __ballot_sync(GPM_FULL_MASK, len > MT_LONG_LIST);
+        for (unsigned m = longs; m; m &= m - 1u) {
+            const int src = __ffs(m) - 1;
+            const int ww = __shfl_sync(GPM_FULL_MASK, w, src), ss = __shfl_sync(GPM_FULL_MASK, sw, src);
+            const int qb = __shfl_sync(GPM_FULL_MASK, b, src), qe = __shfl_sync(GPM_FULL_MASK, e, src);
+            const unsigned exc = __reduce_add_sync(GPM_FULL_MASK, scan(qb + lane, qe, 32, ww, ss));
+            if (lane == 0 && exc) atomicAdd(&E[ss], exc);
+        }
+        for (int i = 0; i < 32 && c0 + i < a1; i += 4) {
+            const int src = i + (lane >> 3);
+            const int ww = __shfl_sync(GPM_FULL_MASK, w, src), ss = __shfl_sync(GPM_FULL_MASK, sw, src);
+            const int qb = __shfl_sync(GPM_FULL_MASK, b, src), qe = __shfl_sync(GPM_FULL_MASK, e, src);
+            unsigned exc = (longs >> src) & 1u ? 0u : scan(qb + (lane & 7), qe, 8, ww, ss);
+            __syncwarp();
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) exc += __shfl_xor_sync(GPM_FULL_MASK, exc, o);
+            if ((lane & 7) == 0 && exc) atomicAdd(&E[ss], exc);
         }
         // these children are done
         __syncwarp();
