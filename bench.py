@@ -849,11 +849,12 @@ def main():
         assert [int(x) for x in c2] == [int(x) for x in counts], "end-to-end counts differ"
     e2e_value = total / (statistics.mean(e2e_ms) / 1000.0)
 
-    # roofline of the dominant kernel (k_clique), an integer-issue-bound
-    # kernel: warp instructions issued per second against the SMs' issue
+    # roofline of the two kernels of the count (k_clique_ne_heavy, which takes
+    # nearly all of the time, and k_clique_ne_light), bound by instruction
+    # issue: warp instructions issued per second against the SMs' issue
     # slots (4 schedulers x 1 instruction per clock per SM), with the
-    # launch's instruction count from the committed ncu summary of the same
-    # launch (identified by its exact word-operation count) and its time
+    # launches' instruction count from the committed ncu summary of the same
+    # launches (identified by their exact word-operation count) and their time
     # measured here; beside it the word operations (AND + POPC of 32-bit
     # candidate words, counted exactly by the kernel) against the POPC rate
     hbm, sm_max, peak_kind = peaks()
@@ -862,23 +863,24 @@ def main():
     peak_ops = sms * POPC_PER_CLK_PER_SM * sm_max * 1e6
     peak_issue = sms * ISSUE_PER_CLK_PER_SM * sm_max * 1e6
     wops = statistics.mean(word_ops)
-    src_hash = kernel_source_hash(["clique.cu", "clique_dev.cuh", "common.cuh"])
-    prof = profiled_launch(f"k_clique_chunglu1m_k{args.k_lo}_{args.k_hi}.txt", src_hash, wops)
+    src_hash = kernel_source_hash(["clique_nonedge.cu", "clique_nonedge.cuh"])
+    summary = f"k_clique_ne_chunglu1m_k{args.k_lo}_{args.k_hi}.txt"
+    prof = profiled_launch(summary, src_hash, wops)
     word_line = {"achieved": wops / kern_s / 1e9, "peak": peak_ops / 1e9,
                  "unit": "Gop/s (32-bit candidate-word AND+POPC)", "frac": wops / kern_s / peak_ops,
                  "peak_kind": f"derived: {sms} SMs x {POPC_PER_CLK_PER_SM} POPC/clk x {sm_max:.0f} MHz",
                  "units_per_launch": wops}
     if prof:
-        roofline = {"bound": "alu", "kernel": "k_clique", "achieved": prof["warp_inst"] / kern_s / 1e9,
+        roofline = {"bound": "alu", "kernel": "k_clique_ne_heavy + k_clique_ne_light", "achieved": prof["warp_inst"] / kern_s / 1e9,
                     "peak": peak_issue / 1e9, "unit": "G warp instructions/s",
                     "frac": prof["warp_inst"] / kern_s / peak_issue,
                     "peak_kind": f"derived: {sms} SMs x {ISSUE_PER_CLK_PER_SM} issue slots/clk x {sm_max:.0f} MHz "
                                  f"({peak_kind} clock)",
                     "units_per_launch": prof["warp_inst"], "traffic": prof["dram_bytes"],
-                    "counts_from": f"profiles/k_clique_chunglu1m_k{args.k_lo}_{args.k_hi}.txt (ncu, same launch)",
+                    "counts_from": f"profiles/{summary} (ncu, same launches)",
                     "word_ops": word_line, "kernel_source_sha": src_hash}
     else:
-        roofline = {"bound": "alu", "kernel": "k_clique", **word_line, "traffic": None,
+        roofline = {"bound": "alu", "kernel": "k_clique_ne_heavy + k_clique_ne_light", **word_line, "traffic": None,
                     "kernel_source_sha": src_hash}
     # HBM: DRAM bytes of the launch (ncu) over its time -- reported beside the
     # ALU roofline to show that memory bandwidth is not what binds the kernel

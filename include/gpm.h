@@ -93,9 +93,11 @@ gpm_status gpm_graph_info(const gpm_graph* g, int32_t* n, int64_t* m, int32_t* m
  * the degree-ordered orientation of G (each clique is reached once, from its
  * lowest-(degree, id) vertex), which plays the role of the paper's "lower"
  * filter.  Roots with at most 1,024 out-neighbours are counted on bitmaps of
- * their out-neighbourhood in shared memory; roots above that, in the same
- * call, by sorted-list intersection (the paper's extension arrays) with
- * per-warp lists in device memory.  out_count: host pointer to one uint64.
+ * their out-neighbourhood in shared memory, branching on the non-edges of the
+ * candidate sets (clique_cpl = 0, a chosen clique_tail or clique_compact, or a
+ * root order other than the default: by walking the cliques instead); roots
+ * above that, in the same call, by sorted-list intersection (the paper's
+ * extension arrays) with per-warp lists in device memory.  out_count: host pointer to one uint64.
  * Errors: GPM_EINVAL, GPM_ENOMEM, GPM_ECUDA, GPM_ETIMEOUT, GPM_EOVERFLOW.
  */
 gpm_status gpm_clique_count(gpm_graph* g, int k, uint64_t* out_count);
@@ -113,9 +115,12 @@ gpm_status gpm_clique_count_range(gpm_graph* g, int k_lo, int k_hi, uint64_t* co
  * motif counting; aggregate_pattern, Section 4.3.4), 1 <= k <=
  * GPM_MOTIF_MAX_K.  counts: host array of counts_len uint64, counts_len >=
  * gpm_motif_num_patterns(k); entry p is the number of subgraphs whose
- * canonical representative is pattern id p (see gpm_motif_pattern).  For
- * k <= 7 the last two levels are counted by entry class (motif_agg_min);
- * k = 8 counts leaf by leaf into global pattern counters.
+ * canonical representative is pattern id p (see gpm_motif_pattern).  k = 3 .. 5
+ * on graphs of at most 2^14 vertices and degree 2^10, and k = 3, 4 on larger
+ * ones, come from homomorphism counts (motif_agg_min = 0, or a root order other
+ * than the default: from the walk over the sets); otherwise the walk counts
+ * the last two levels by entry class for k <= 7 (motif_agg_min), and k = 8 leaf
+ * by leaf into global pattern counters.
  * Errors: GPM_EINVAL (also counts_len too small), GPM_ENOMEM, GPM_ECUDA,
  * GPM_ETIMEOUT, GPM_EOVERFLOW.
  */
@@ -177,7 +182,8 @@ typedef struct {
                                /* rows get shorter, 2 whenever they get shorter                     */
     int32_t motif_agg_min;     /* motif: a node one level above the leaves whose extension array     */
                                /* has at least this many entries left counts its last two levels by  */
-                               /* entry class instead of leaf by leaf (0: never)                     */
+                               /* entry class instead of leaf by leaf (0: never, and whole-graph     */
+                               /* counts of k <= 5 walk the sets too)                                 */
     int32_t clique_compact3;   /* three-level clique tail on the node's members whenever that        */
                                /* shortens the rows: 0 never, 1 (default), 2 also with the pairs of  */
                                /* nodes of at most 64 members taken one at a time by the whole warp  */
@@ -189,7 +195,8 @@ typedef struct {
                                /* sum_t C(a_t, 2) minus the open wedges found from the non-edges,     */
                                /* instead of one AND + POPC per (k-1)-clique: 0 never, 1 always,      */
                                /* 2..100 for tail nodes whose members are at least this percent       */
-                               /* pairwise adjacent (default 85)                                      */
+                               /* pairwise adjacent (default 85); 0 also makes whole-graph counts     */
+                               /* walk the cliques                                                    */
 } gpm_config;
 
 #define GPM_ORDER_ID          0  /* roots in id order                               */
@@ -202,7 +209,7 @@ gpm_status gpm_set_config(gpm_graph* g, const gpm_config* cfg);
 /* Statistics of the last counting call on g (device-measured). */
 typedef struct {
     double   kernel_ms;        /* enumeration kernel time (CUDA events)          */
-    uint64_t units_done;       /* work units (roots + donated units) finished     */
+    uint64_t units_done;       /* work units (roots, or vertices, + donated units) finished */
     uint64_t donations;        /* units handed to idle warps (work donation)      */
     uint64_t idle_polls;       /* spins of idle warps waiting for a hand-off      */
     int32_t  grid_blocks;      /* persistent grid size                            */
