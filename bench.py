@@ -3,10 +3,10 @@
 Default workload (the plain method at scale): k-clique counting on the
 Chung-Lu power-law graph (n = 1,000,000, average degree 16, exponent 2.1,
 expected degrees capped at 20,000, seed 1), degree-ordered, int32 CSR.  One
-step = one enumeration that counts every clique size 4..7
+step = one call that counts every clique size 4..7
 (gpm_clique_count_range), with the graph already resident in HBM.  The
-configuration's full range 4..8 is one enumeration of about half a minute:
-it is timed once, beside the steps, as the ``k4_8`` entry.
+configuration's full range 4..8 is timed once, beside the steps, as the
+``k4_8`` entry.
 
 Beside the headline the line carries one timed, oracle-checked entry per
 workload of the method (``configs``): 4-vertex motifs on a 516-vertex
@@ -548,7 +548,8 @@ def balancing_ablation(stream, full: bool = False) -> dict:
     host-monitored stop / redistribute / restart (thresholds 40 % for
     cliques and 10 % for motifs, the paper's best), and no balancing at
     all.  Workloads: chunglu1m 7-cliques (the headline's deepest size) and
-    sbm2000 5-motifs."""
+    sbm2000 5-motifs, both by the walk over every root, heaviest first (the
+    whole-graph calls need no balancing)."""
     from paper_2212_04551_gb300 import gpm
     from paper_2212_04551_gb300 import graphs as G
     out = {}
@@ -556,11 +557,9 @@ def balancing_ablation(stream, full: bool = False) -> dict:
         g = G.workload(name)
         dg = gpm.graph_from_csr(g, stream=stream)
         res = {}
-        if app == gpm.GPM_APP_CLIQUE:
-            ref, ms = timed(lambda: gpm.gpm_clique_count(dg, k), stream)
-            ref = np.array([ref], dtype=np.uint64)
-        else:
-            ref, ms = timed(lambda: gpm.gpm_motif_count(dg, k), stream)
+        roots = (heaviest_first(g) if app == gpm.GPM_APP_CLIQUE
+                 else np.argsort(-g.degrees(), kind="stable").astype(np.int32))
+        (ref, _), ms = timed(lambda: gpm.gpm_count_roots(dg, app, k, roots), stream)
         st = gpm.gpm_get_stats(dg)
         res["in_kernel_handoff"] = {"ms": ms, "kernel_ms": st["kernel_ms"], "idle_warp_frac": st["idle_warp_frac"],
                                     "handoffs": int(st["donations"])}
@@ -571,7 +570,7 @@ def balancing_ablation(stream, full: bool = False) -> dict:
         res["speedup_handoff_vs_monitored"] = res["host_monitored"]["ms"] / res["in_kernel_handoff"]["ms"]
         if full or app != gpm.GPM_APP_CLIQUE:
             gpm.gpm_set_config(dg, donate=0)
-            c = gpm.gpm_clique_count(dg, k) if app == gpm.GPM_APP_CLIQUE else gpm.gpm_motif_count(dg, k)
+            c = gpm.gpm_count_roots(dg, app, k, roots)[0]
             st = gpm.gpm_get_stats(dg)
             res["none"] = {"kernel_ms": st["kernel_ms"], "idle_warp_frac": st["idle_warp_frac"],
                            "same_counts": bool(np.array_equal(np.ravel(c), np.ravel(ref)))}
@@ -583,7 +582,7 @@ def balancing_ablation(stream, full: bool = False) -> dict:
 
 def dm_dfs_ablation(stream, full: bool = False) -> dict:
     """The paper's DM_DFS baseline (one thread per root, sorted-list merges,
-    no balancing) against the warp-centric bitmap kernel with hand-offs, on
+    no balancing) against the warp-centric bitmap walk with hand-offs, on
     chunglu1m cliques k = 4 and 5 (the paper's Table optimizations-
     performance compares its DFS and warp-centric forms the same way)."""
     from paper_2212_04551_gb300 import gpm
@@ -592,6 +591,7 @@ def dm_dfs_ablation(stream, full: bool = False) -> dict:
     dg = gpm.graph_from_csr(g, stream=stream)
     out = {}
     for k in ((4, 5) if full else (4,)):
+        gpm.gpm_set_config(dg, clique_cpl=0)      # the walk, not the branching on non-edges
         c = gpm.gpm_clique_count(dg, k)
         wc = gpm.gpm_get_stats(dg)["kernel_ms"]
         cd = gpm.gpm_clique_count_dfs(dg, k)
