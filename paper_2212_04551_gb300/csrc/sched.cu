@@ -95,8 +95,13 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_root(const int32_t* __restr
 // Bound: the barriers, about one per round and level.  Up to CORE_CLUSTER_N
 // vertices the launch is one cluster of eight blocks, whose barrier is a
 // hardware one; above, one block per SM (the scans of a level need the threads).
-// One launch per pass over all vertices, with the host reading a flag in
-// between, took 55 us a pass: 10.2 ms on rmat14 (185 passes).
+// Between two barriers a round is a chain of dependent loads, so each lane
+// keeps four entries in flight and a short round spreads each list over up to a
+// block (eight lanes per vertex left a hub's list serial), and the last level
+// ends without its round: its vertices lower nothing.
+// All root features: R-MAT 2^14 2.1 -> 0.87 ms, 2^16 4.9 -> 2.25, 10^6-vertex
+// Chung-Lu 62 -> 15.9.  One launch per pass over all vertices, with the host
+// reading a flag in between, took 9.4, 16.4 and 254 ms.
 constexpr int CORE_THREADS = 512;
 constexpr int CORE_CLUSTER = 8;
 constexpr int CORE_CLUSTER_N = 1 << 17;
@@ -131,14 +136,24 @@ __global__ void __launch_bounds__(CORE_THREADS) k_core(const int32_t* __restrict
     for (;;) {
         // the vertices of level c, and the smallest degree above it
         int least = INT32_MAX;
-        for (long long v = tid; v < n; v += nt) {
-            if (core[v] >= 0) continue;
-            const int r = rem[v];
-            if (r <= c) {
-                core[v] = c;
-                (round & 1 ? queue1 : queue0)[atomicAdd(&st->n_queue[round % 3], 1)] = (int32_t)v;
-            } else {
-                least = min(least, r);
+        for (long long v0 = tid; v0 < n; v0 += 4 * nt) {
+            int cs[4], rs[4];
+#pragma unroll
+            for (int z = 0; z < 4; z++) {
+                const long long v = v0 + z * nt;
+                cs[z] = v < n ? core[v] : 0;
+                rs[z] = v < n ? rem[v] : 0;
+            }
+#pragma unroll
+            for (int z = 0; z < 4; z++) {
+                if (cs[z] >= 0) continue;
+                const long long v = v0 + z * nt;
+                if (rs[z] <= c) {
+                    core[v] = c;
+                    (round & 1 ? queue1 : queue0)[atomicAdd(&st->n_queue[round % 3], 1)] = (int32_t)v;
+                } else {
+                    least = min(least, rs[z]);
+                }
             }
         }
         least = (int)__reduce_min_sync(GPM_FULL_MASK, (unsigned)least);
@@ -148,28 +163,40 @@ __global__ void __launch_bounds__(CORE_THREADS) k_core(const int32_t* __restrict
         const bool none = *(volatile int*)&st->n_queue[round % 3] == 0;
         if (tid == 0) st->min_left[(scan + 1) & 1] = INT32_MAX;
         scan++;
+        if (left == INT32_MAX) break;    // every vertex that was left has level c: nothing to lower
         for (;;) {
             const int m = *(volatile int*)&st->n_queue[round % 3];
             if (!m) break;
             const int32_t* q = round & 1 ? queue1 : queue0;
             int32_t* next = round & 1 ? queue0 : queue1;
-            // eight lanes per removed vertex
-            for (long long i = tid >> 3; i < m; i += nt >> 3) {
+            // 2^sh lanes per removed vertex: at least eight, more while the round
+            // leaves threads over, at most a block (a divisor of the thread count)
+            int sh = 3;
+            while ((2 << sh) <= CORE_THREADS && ((long long)m << (sh + 1)) <= nt) sh++;
+            const int w = 1 << sh;
+            for (long long i = tid >> sh; i < m; i += nt >> sh) {
                 const int v = __ldcg(q + i);
-                for (int t = indptr[v] + (int)(tid & 7), e = indptr[v + 1]; t < e; t += 8) {
-                    const int u = indices[t];
-                    if (*(volatile int*)&core[u] >= 0) continue;
-                    if (atomicSub(&rem[u], 1) == c + 1) {
-                        *(volatile int*)&core[u] = c;
-                        next[atomicAdd(&st->n_queue[(round + 1) % 3], 1)] = u;
-                    }
+                const long long e = indptr[v + 1];
+                for (long long t = indptr[v] + (tid & (w - 1)); t < e; t += 4 * w) {
+                    int us[4], old[4];
+#pragma unroll
+                    for (int z = 0; z < 4; z++) us[z] = t + z * w < e ? indices[t + z * w] : -1;
+#pragma unroll
+                    for (int z = 0; z < 4; z++) old[z] = us[z] < 0 ? 0 : *(volatile int*)&core[us[z]];
+#pragma unroll
+                    for (int z = 0; z < 4; z++) old[z] = old[z] < 0 ? atomicSub(&rem[us[z]], 1) : -1;
+#pragma unroll
+                    for (int z = 0; z < 4; z++)
+                        if (old[z] == c + 1) {
+                            *(volatile int*)&core[us[z]] = c;
+                            next[atomicAdd(&st->n_queue[(round + 1) % 3], 1)] = us[z];
+                        }
                 }
             }
             if (tid == 0) st->n_queue[(round + 2) % 3] = 0;
             core_sync<CLUSTER>();
             round++;
         }
-        if (left == INT32_MAX) break;    // every vertex had level <= c
         // (the rounds of level c can have brought vertices down to c + 1)
         c = none ? left : c + 1;
         core_sync<CLUSTER>();
