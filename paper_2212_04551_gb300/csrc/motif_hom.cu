@@ -436,13 +436,15 @@ __global__ void k_hom_edges(const int32_t* __restrict__ indptr, const int32_t* _
 
 // thread per (graph, pattern)
 __global__ void k_hom_finish(const unsigned long long* __restrict__ hom, long long n_out, int npat,
-                             const long long* __restrict__ coef, unsigned long long* __restrict__ out) {
+                             const long long* __restrict__ coef, unsigned long long* __restrict__ out, int clique_hom,
+                             int clique_aut, unsigned long long* __restrict__ clique_out) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_out; i += (long long)gridDim.x * blockDim.x) {
         const long long g = i / npat, pat = i % npat;
         const unsigned long long* h = hom + g * HOM_N;
         unsigned long long sum = 0;
         for (int j = 0; j < HOM_N; j++) sum += (unsigned long long)coef[pat * HOM_N + j] * h[j];
         out[i] = sum / (unsigned long long)coef[(long long)npat * HOM_N + pat];
+        if (clique_out && pat == 0) clique_out[g] = h[clique_hom] / (unsigned)clique_aut;
     }
 }
 
@@ -558,12 +560,16 @@ void hom_combine(const HomTable& t, const unsigned long long* hom, uint64_t* cou
     }
 }
 
-cudaError_t launch_hom_finish(const unsigned long long* hom, int n_graphs, int k, unsigned long long* out, cudaStream_t s) {
+cudaError_t launch_hom_finish(const unsigned long long* hom, int n_graphs, int k, unsigned long long* out, int clique_k,
+                              unsigned long long* clique_out, cudaStream_t s) {
     const int npat = hom_table(k).npat;
     const long long n_out = (long long)n_graphs * npat;
     if (n_out <= 0) return cudaSuccess;
     const long long* coef = device_hom_table(k);
-    k_hom_finish<<<(int)std::min<long long>((n_out + 255) / 256, 1024), 256, 0, s>>>(hom, n_out, npat, coef, out);
+    const int clique_hom = clique_k == 3 ? H_TRI : clique_k == 4 ? H_K4 : H_K5;
+    const int clique_aut = clique_k == 3 ? 6 : clique_k == 4 ? 24 : 120;      // every clique is hit k! times
+    k_hom_finish<<<(int)std::min<long long>((n_out + 255) / 256, 1024), 256, 0, s>>>(
+        hom, n_out, npat, coef, out, clique_hom, clique_aut, clique_k > 0 ? clique_out : nullptr);
     return cudaGetLastError();
 }
 

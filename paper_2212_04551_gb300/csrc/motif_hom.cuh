@@ -72,7 +72,9 @@ void run_motif_hom(gpm_graph* g, int k, uint64_t* counts_out);
 // Larger graphs, k = 3 and 4 (motif_sparse.cu; builds the orientation)
 bool motif_sparse_applies(gpm_graph* g, int k);
 void run_motif_sparse(gpm_graph* g, int k, uint64_t* counts_out);
-// out[g * npat + p] = count of pattern p in graph g
-cudaError_t launch_hom_finish(const unsigned long long* hom, int n_graphs, int k, unsigned long long* out, cudaStream_t s);
+// out[g * npat + p] = count of pattern p in graph g; clique_k > 0 (at most k): the
+// cliques of that size of every graph as well, from the same sums
+cudaError_t launch_hom_finish(const unsigned long long* hom, int n_graphs, int k, unsigned long long* out, int clique_k,
+                              unsigned long long* clique_out, cudaStream_t s);
 
 }  // namespace gpm

@@ -83,3 +83,16 @@ def test_larger_graphs_against_the_walk(name, k):
     assert np.array_equal(ours, gpm.gpm_count_roots(dg, gpm.GPM_APP_MOTIF, k)[0])
     gpm.gpm_set_config(dg, motif_agg_min=0)
     assert np.array_equal(ours, gpm.gpm_motif_count(dg, k))
+
+
+@pytest.mark.parametrize("kc,km", [(3, 3), (3, 5), (4, 4), (4, 5), (5, 5), (5, 4), (6, 5)])
+def test_batched_cliques_from_the_same_sums(kc, km):
+    """Cliques no larger than the motifs share their sums; the others, and the
+    walk's form of the call, keep units of their own."""
+    gs = [make() for make in GRAPHS.values()] + [G.empty(0), G.empty(1), G.complete(40)]
+    b = gpm.batch_from_graphs(gs)
+    cliques, motifs = gpm.gpm_batch_count(b, kc, km)
+    assert [int(c) for c in cliques] == [O.clique_count(g, kc) for g in gs]
+    gpm.gpm_batch_set_config(b, motif_agg_min=0)
+    walked = gpm.gpm_batch_count(b, kc, km)
+    assert np.array_equal(cliques, walked[0]) and np.array_equal(motifs, walked[1])
