@@ -330,7 +330,7 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     p.n_units = n_units;
     p.kc = kc;
     p.km = km;
-    p.lut = km > 0 ? device_lut(km) : nullptr;
+    p.lut = km > 0 ? device_lut(km, b->stream) : nullptr;
     if (kc > 0 && g->max_outdeg > 1024) fail(GPM_ENOTIMPL, "batched clique counting needs out-degrees <= 1024");
     p.cq_maxd = std::max(kc > 0 ? g->max_outdeg : 1, 1);
     p.cq_wmax = (p.cq_maxd + 31) / 32;
@@ -402,7 +402,7 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
         hp.ctl = p.ctl;
         if (hom_k == 5) hp.edges = ensure_hom_edges(g, hp.goff, hp.vgraph);
         hgr = plan_hom(hp, hom_k, g->num_sms);
-        device_hom_table(hom_k);
+        device_hom_table(hom_k, b->stream);
         if (n_units == 0) {
             c.blocks = hgr.blocks;
             c.wpb = hgr.warps_per_block;

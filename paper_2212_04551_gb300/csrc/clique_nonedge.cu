@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(NE_WARPS * 32, DEEP ? 5 : 10) k_clique_ne_heav
 // ------------------------------------------------------------------- host
 
 // C(n, k), saturated, on the current device (uploaded once per device)
-static const unsigned long long* device_binomials() {
+static const unsigned long long* device_binomials(cudaStream_t s) {
     static std::mutex mu;
     static std::map<int, unsigned long long*> tables;
     int dev = 0;
@@ -586,17 +586,7 @@ static const unsigned long long* device_binomials() {
                 x = a + b < a || a == ~0ull || b == ~0ull ? ~0ull : a + b;
             }
         }
-    unsigned long long* d = nullptr;
-    const size_t bytes = t.size() * sizeof(unsigned long long);
-    if (cudaMalloc(&d, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        fail(GPM_ENOMEM, "cudaMalloc for the binomial table failed");
-    }
-    const cudaError_t e = cudaMemcpy(d, t.data(), bytes, cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-        cudaFree(d);
-        check_cuda(e, "cudaMemcpy(binomial table)");
-    }
+    auto* d = static_cast<unsigned long long*>(upload_table(t.data(), t.size() * sizeof(t[0]), s, "binomial table"));
     tables[dev] = d;
     return d;
 }
@@ -614,7 +604,7 @@ int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* 
     p.deg = g->degree.as<int32_t>();
     p.ne.k_lo = std::max(k_lo, 3);
     p.ne.k_hi = k_hi;
-    p.ne.binom = device_binomials();
+    p.ne.binom = device_binomials(s);
     p.ctl = ctl;
     p.tri = tri;
     // positions by out-degree: [0, above) list path, [above, big) heavy, [big, all) light

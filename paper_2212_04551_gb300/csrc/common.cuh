@@ -174,6 +174,9 @@ void ensure_dag(gpm_graph* g);
 const int32_t* ensure_root_order(gpm_graph* g, int app);  // plain scheduler order
 const int32_t* ensure_id_order(gpm_graph* g);             // 0, 1, ..., n-1
 long long roots_at_least(gpm_graph* g, int d);            // vertices of out-degree >= d: the first ones of the clique order
+// A table of the process's lifetime on the current device, from host memory, on
+// stream s; it is there when the call returns, for launches on any stream.
+void* upload_table(const void* host, size_t bytes, cudaStream_t s, const char* what);
 void exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, int64_t* total,
                         cudaStream_t s, DevBuf& tmp);
 
@@ -185,7 +188,7 @@ struct PatternTable {
     std::vector<uint16_t> lut;            // traversal code -> pattern id (0xFFFF invalid)
 };
 const PatternTable& pattern_table(int k);  // built once per k, cached
-const uint16_t* device_lut(int k);         // uploaded once per (device, k)
+const uint16_t* device_lut(int k, cudaStream_t s);   // uploaded once per (device, k), on s
 
 // Pre-split of a schedule's split roots (positions n_counter .. n_roots-1 of
 // the root list): root j becomes units d_chunk_off[j] .. d_chunk_off[j+1]-1

@@ -64,6 +64,24 @@ void DevBuf::ensure(size_t need) {
     bytes = want;
 }
 
+// A copy from pageable memory may return before it has reached the device, and
+// a non-blocking stream is not ordered behind the legacy one: hence the stream
+// of the caller, and the wait.
+void* upload_table(const void* host, size_t bytes, cudaStream_t s, const char* what) {
+    void* d = nullptr;
+    if (cudaMalloc(&d, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        fail(GPM_ENOMEM, std::string("cudaMalloc for the ") + what + " failed");
+    }
+    cudaError_t e = cudaMemcpyAsync(d, host, bytes, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+        cudaFree(d);
+        check_cuda(e, what);
+    }
+    return d;
+}
+
 // --------------------------------------------------------------- kernels
 
 // Ids in range, no self-loop, strictly ascending, and the reverse edge present

@@ -143,7 +143,7 @@ const PatternTable& pattern_table(int k) {
 static std::mutex g_dlut_mu;
 static std::map<std::pair<int, int>, uint16_t*> g_dluts;  // (device, k) -> device table (process lifetime)
 
-const uint16_t* device_lut(int k) {
+const uint16_t* device_lut(int k, cudaStream_t s) {
     const PatternTable& t = pattern_table(k);
     int dev = 0;
     check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
@@ -151,14 +151,7 @@ const uint16_t* device_lut(int k) {
     auto key = std::make_pair(dev, k);
     auto it = g_dluts.find(key);
     if (it != g_dluts.end()) return it->second;
-    uint16_t* d = nullptr;
-    const size_t bytes = t.lut.size() * sizeof(uint16_t);
-    cudaError_t e = cudaMalloc(&d, bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        fail(GPM_ENOMEM, "cudaMalloc for the pattern table failed");
-    }
-    check_cuda(cudaMemcpy(d, t.lut.data(), bytes, cudaMemcpyHostToDevice), "cudaMemcpy(pattern table)");
+    auto* d = static_cast<uint16_t*>(upload_table(t.lut.data(), t.lut.size() * sizeof(uint16_t), s, "pattern table"));
     g_dluts[key] = d;
     return d;
 }

@@ -383,7 +383,7 @@ void run_motif(gpm_graph* g, int k, const int32_t* d_roots, int64_t n_roots,
         return;
     }
 
-    const uint16_t* lut = device_lut(k);
+    const uint16_t* lut = device_lut(k, s);
 
     MotifParams p{};
     p.indptr = g->indptr.as<int32_t>();

@@ -565,7 +565,7 @@ cudaError_t launch_hom_finish(const unsigned long long* hom, int n_graphs, int k
     const int npat = hom_table(k).npat;
     const long long n_out = (long long)n_graphs * npat;
     if (n_out <= 0) return cudaSuccess;
-    const long long* coef = device_hom_table(k);
+    const long long* coef = device_hom_table(k, s);
     const int clique_hom = clique_k == 3 ? H_TRI : clique_k == 4 ? H_K4 : H_K5;
     const int clique_aut = clique_k == 3 ? 6 : clique_k == 4 ? 24 : 120;      // every clique is hit k! times
     k_hom_finish<<<(int)std::min<long long>((n_out + 255) / 256, 1024), 256, 0, s>>>(
@@ -727,7 +727,7 @@ const HomTable& hom_table(int k) {
     return tables[k] = std::move(t);
 }
 
-const long long* device_hom_table(int k) {
+const long long* device_hom_table(int k, cudaStream_t s) {
     static std::mutex mu;
     static std::map<std::pair<int, int>, long long*> tables;
     const HomTable& t = hom_table(k);
@@ -738,16 +738,7 @@ const long long* device_hom_table(int k) {
     if (it != tables.end()) return it->second;
     std::vector<long long> both(t.coef);
     both.insert(both.end(), t.aut.begin(), t.aut.end());
-    long long* d = nullptr;
-    if (cudaMalloc(&d, both.size() * sizeof(long long)) != cudaSuccess) {
-        cudaGetLastError();
-        fail(GPM_ENOMEM, "cudaMalloc for the homomorphism table failed");
-    }
-    const cudaError_t e = cudaMemcpy(d, both.data(), both.size() * sizeof(long long), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-        cudaFree(d);
-        check_cuda(e, "cudaMemcpy(homomorphism table)");
-    }
+    auto* d = static_cast<long long*>(upload_table(both.data(), both.size() * sizeof(both[0]), s, "homomorphism table"));
     return tables[{dev, k}] = d;
 }
 

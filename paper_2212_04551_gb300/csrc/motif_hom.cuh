@@ -28,7 +28,7 @@ struct HomTable {
 };
 const HomTable& hom_table(int k);                 // host, built once per k
 void hom_combine(const HomTable& t, const unsigned long long* hom, uint64_t* counts_out);
-const long long* device_hom_table(int k);         // coef, then aut; uploaded once per device
+const long long* device_hom_table(int k, cudaStream_t s);   // coef, then aut; uploaded once per device, on s
 
 struct HomLaunch {
     const int32_t* __restrict__ indptr;

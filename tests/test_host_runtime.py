@@ -1,0 +1,51 @@
+"""The library's host code on a stand-in CUDA runtime (fake_gpu.py): the order
+of copies and launches, failing calls, limits.  CPU only."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from fake_gpu import link
+from paper_2212_04551_gb300 import gpm
+
+
+@pytest.fixture(scope="module")
+def _linked(tmp_path_factory):
+    # a library of its own per test module: tables are uploaded once per process
+    return link(tmp_path_factory.mktemp("fake"))
+
+
+@pytest.fixture
+def gpu(_linked):
+    _linked.lib.fake_reset()
+    return _linked
+
+
+def _path(n):
+    """A path's CSR, n >= 2."""
+    indptr = np.r_[0, 1, np.arange(3, 2 * n - 2, 2), 2 * n - 2]
+    indices = np.ravel(np.c_[np.arange(n) - 1, np.arange(n) + 1])[1:-1]
+    return indptr, indices
+
+
+def _two_paths(n):
+    ip, ix = _path(n)
+    return [0, n, 2 * n], np.r_[ip, ip[-1] + ip[1:]], np.r_[ix, ix + n]
+
+
+@pytest.mark.parametrize("what", ["binomials", "patterns", "batch"])
+def test_tables_have_landed_before_a_launch_on_another_stream(gpu, what):
+    """The tables come from pageable memory, whose copy may still be in flight
+    when the call returns, and a non-blocking stream waits for no other."""
+    if what == "batch":
+        b = gpu.batch(*_two_paths(20))            # on a non-blocking stream of its own
+        assert gpu.batch_count(b, 0, 5, 2) == gpm.GPM_OK, gpu.error()     # homomorphism table
+        assert gpu.batch_count(b, 0, 6, 2) == gpm.GPM_OK, gpu.error()     # pattern table
+        gpu.lib.gpm_batch_destroy(b)
+    else:
+        n, k = (20000, 4) if what == "binomials" else (40, 7)
+        g = gpu.graph(*_path(n), stream=gpu.lib.fake_stream(1))
+        assert gpu.motifs(g, k) == gpm.GPM_OK, gpu.error()
+        gpu.lib.gpm_graph_destroy(g)
+    assert gpu.log()
+    assert gpu.lib.fake_violations() == 0
