@@ -33,6 +33,7 @@
 #include <map>
 #include <string>
 #include <tuple>
+#include <utility>
 #include <vector>
 
 #include "clique_dev.cuh"
@@ -63,6 +64,15 @@ struct gpm_batch {
         unsigned long long* host_out = nullptr;   // pinned
         size_t words = 0;
         int blocks = 0, wpb = 0, launches = 0;
+        Captured() = default;
+        Captured(Captured&& o) noexcept
+            : exec(std::exchange(o.exec, nullptr)), units(std::move(o.units)), uranges(std::move(o.uranges)),
+              dev_out(std::move(o.dev_out)), dev_hom(std::move(o.dev_hom)), host_out(std::exchange(o.host_out, nullptr)),
+              words(o.words), blocks(o.blocks), wpb(o.wpb), launches(o.launches) {}
+        ~Captured() {
+            if (exec) cudaGraphExecDestroy(exec);
+            if (host_out) cudaFreeHost(host_out);
+        }
     };
     // (kc, km, wpb, bps, order, motif_agg_min, batch_split)
     std::map<std::tuple<int, int, int, int, int, int, int>, Captured> graphs;
@@ -364,21 +374,18 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     if (bps > 0) per_sm = std::min(per_sm, bps);
     const int blocks = per_sm * g->num_sms;
 
-    gpm_batch::Captured& c = b->graphs[key];
+    // (the entry goes into the map when it can be launched: a call that fails on
+    // the way leaves nothing behind, and the next one tries again)
+    gpm_batch::Captured c;
     c.units = std::move(units);
     c.uranges = std::move(uranges);
     const size_t G = (size_t)b->n_graphs;
     const size_t ctl_words = (sizeof(Control) + 7) / 8;
     c.words = G + G * npat + ctl_words;
     const size_t hom_bytes = sizeof(unsigned long long) * (G * HOM_N + 1);
-    try {
-        if (hom) c.dev_hom.ensure(hom_bytes);
-        c.dev_out.ensure(sizeof(unsigned long long) * c.words);
-        GPM_CUDA(cudaMallocHost(&c.host_out, sizeof(unsigned long long) * c.words));
-    } catch (...) {
-        b->graphs.erase(key);
-        throw;
-    }
+    if (hom) c.dev_hom.ensure(hom_bytes);
+    c.dev_out.ensure(sizeof(unsigned long long) * c.words);
+    GPM_CUDA(cudaMallocHost(&c.host_out, sizeof(unsigned long long) * c.words));
     p.clique_out = c.dev_out.as<unsigned long long>();
     p.motif_out = p.clique_out + G;
     p.ctl = reinterpret_cast<Control*>(p.motif_out + G * npat);
@@ -428,18 +435,12 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     cudaError_t e2 = cudaStreamEndCapture(b->stream, &graph);
     if (e1 != cudaSuccess || e2 != cudaSuccess) {
         if (graph) cudaGraphDestroy(graph);
-        cudaFreeHost(c.host_out);
-        b->graphs.erase(key);
         check_cuda(e1 != cudaSuccess ? e1 : e2, "CUDA graph capture of the batched launch");
     }
     cudaError_t e3 = cudaGraphInstantiate(&c.exec, graph, 0);
     cudaGraphDestroy(graph);
-    if (e3 != cudaSuccess) {
-        cudaFreeHost(c.host_out);
-        b->graphs.erase(key);
-        check_cuda(e3, "cudaGraphInstantiate");
-    }
-    return c;
+    check_cuda(e3, "cudaGraphInstantiate");
+    return b->graphs.emplace(key, std::move(c)).first->second;
 }
 
 // One replay; results in cap.host_out.  Returns the device time (ms).
@@ -536,10 +537,6 @@ gpm_batch* create_batch(const int32_t* graph_off, const int32_t* indptr, const i
 void destroy_batch(gpm_batch* b) {
     if (!b) return;
     if (b->stream) cudaStreamSynchronize(b->stream);
-    for (auto& kv : b->graphs) {
-        if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
-        if (kv.second.host_out) cudaFreeHost(kv.second.host_out);
-    }
     b->graphs.clear();
     b->g->stream = nullptr;
     destroy_graph(b->g);

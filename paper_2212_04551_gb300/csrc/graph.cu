@@ -36,6 +36,7 @@ const char* last_error_cstr() { return t_last_error.c_str(); }
 
 void check_cuda(cudaError_t e, const char* what) {
     if (e == cudaSuccess) return;
+    cudaGetLastError();   // reported here, not by the next call's launch check
     gpm_status s = (e == cudaErrorMemoryAllocation) ? GPM_ENOMEM : GPM_ECUDA;
     fail(s, std::string(what) + ": " + cudaGetErrorString(e));
 }

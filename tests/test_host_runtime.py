@@ -49,3 +49,26 @@ def test_tables_have_landed_before_a_launch_on_another_stream(gpu, what):
         gpu.lib.gpm_graph_destroy(g)
     assert gpu.log()
     assert gpu.lib.fake_violations() == 0
+
+
+@pytest.mark.parametrize("kc,km", [(4, 5), (5, 4), (4, 6), (3, 0)])
+def test_a_failed_first_batch_call_leaves_nothing_behind(gpu, kc, km):
+    """Whatever allocation (or step of the capture) fails in a batch's first
+    call, the next one tries again and succeeds, and nothing is leaked."""
+    warm = gpu.batch(*_two_paths(20))                       # the tables of the process
+    assert gpu.batch_count(warm, kc, km, 2) == gpm.GPM_OK, gpu.error()
+    gpu.lib.gpm_batch_destroy(warm)
+    before = gpu.lib.fake_memory_in_use()
+    for at in range(1, 100):
+        b = gpu.batch(*_two_paths(20))
+        gpu.lib.fake_fail(b"alloc", at)
+        st = gpu.batch_count(b, kc, km, 2)
+        failed = gpu.lib.fake_failed()
+        assert st == (gpm.GPM_ENOMEM if failed else gpm.GPM_OK), (at, gpu.error())
+        gpu.lib.fake_fail(b"", 0)
+        assert gpu.batch_count(b, kc, km, 2) == gpm.GPM_OK, (at, gpu.error())
+        gpu.lib.gpm_batch_destroy(b)
+        assert gpu.lib.fake_memory_in_use() == before, at
+        if not failed:
+            break
+    assert at > 3 and not failed
