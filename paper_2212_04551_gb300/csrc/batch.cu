@@ -368,7 +368,7 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     size_t smem = layout(hom_k);
     if (smem > 227 * 1024) fail(GPM_ENOTIMPL, "batched state does not fit in shared memory (graphs too large)");
     if (hom) smem = layout(0);
-    GPM_CUDA(cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    allow_shared((const void*)k_batch, smem);
     int per_sm = resident_blocks((const void*)k_batch, wpb * 32, smem);
     if (per_sm <= 0) fail(GPM_EINVAL, "batched kernel cannot be resident with this configuration");
     if (bps > 0) per_sm = std::min(per_sm, bps);

@@ -343,7 +343,7 @@ static CliqueLaunch plan_clique_launch(gpm_graph* g, int k_lo, int k_hi, const i
         smem = (size_t)wpb * L.total * 4;
     }
     if (smem > 227 * 1024) fail(GPM_ENOTIMPL, "clique bitmap does not fit in shared memory");
-    GPM_CUDA(cudaFuncSetAttribute(k_clique, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    allow_shared((const void*)k_clique, smem);
     c.gr = plan_grid(g, (const void*)k_clique, wpb, smem);
     c.wpb = wpb;
     c.smem = smem;

@@ -632,7 +632,7 @@ int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* 
         p.ticket = tickets;
         p.next_child = reinterpret_cast<unsigned int*>(tickets + 32);
         const size_t smem = 4 * ((size_t)ne_block_words(p.maxd, p.ws) + (size_t)NE_WARPS * p.warp_words);
-        GPM_CUDA(cudaFuncSetAttribute(heavy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        allow_shared(heavy, smem);
         Grid gr = plan_grid(g, heavy, NE_WARPS, smem);
         gr.blocks = (int)std::min<long long>(gr.blocks, n_big + p.n_help * p.rounds);
         if (deep) k_clique_ne_heavy<true><<<gr.blocks, NE_WARPS * 32, smem, s>>>(p);

@@ -254,6 +254,7 @@ void order_by_score(gpm_graph* g, const float* d_score, const int32_t* d_roots, 
 
 // helpers
 int resident_blocks(const void* kernel, int threads, size_t smem);
+void allow_shared(const void* kernel, size_t bytes);   // dynamic shared memory that launches of the kernel may ask for
 // max_per_sm > 0 caps the resident blocks per SM unless the configuration sets blocks_per_sm
 Grid plan_grid(gpm_graph* g, const void* kernel, int warps_per_block, size_t smem_per_block, int max_per_sm = 0);
 // warps per block (16, 8, 4, 2 or 1) that keeps the most warps resident per SM

@@ -16,8 +16,10 @@
 #include <algorithm>
 #include <climits>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -552,14 +554,27 @@ int resident_blocks(const void* kernel, int threads, size_t smem) {
     return nb;
 }
 
+// The attribute belongs to the kernel, not to the call: it only grows, so that a
+// call on a smaller graph cannot lower it between another thread's plan and
+// launch (or below what a captured launch needs).
+void allow_shared(const void* kernel, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, size_t> most;
+    int dev = 0;
+    GPM_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    size_t& m = most[{dev, kernel}];
+    const size_t want = std::max(m, bytes);
+    GPM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want));
+    m = want;
+}
+
 int best_warps_per_block(const void* kernel, size_t smem_per_warp, size_t smem_fixed) {
     int best = 8, best_warps = -1;
     for (int wpb : {16, 8, 4, 2, 1}) {
         const size_t smem = smem_fixed + smem_per_warp * wpb;
         if (smem > 227 * 1024) continue;
-        if (smem > 48 * 1024)
-            check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                       "cudaFuncSetAttribute");
+        if (smem > 48 * 1024) allow_shared(kernel, smem);
         const int per_sm = resident_blocks(kernel, wpb * 32, smem);
         if (per_sm * wpb > best_warps) {
             best_warps = per_sm * wpb;

@@ -444,7 +444,7 @@ void run_motif(gpm_graph* g, int k, const int32_t* d_roots, int64_t n_roots,
     const void* kfun = list ? (smem_state ? (const void*)k_motif<true, true, true> : (const void*)k_motif<false, true, true>)
                        : smem_state ? (gcount ? (const void*)k_motif<true, true> : (const void*)k_motif<true, false>)
                                     : (gcount ? (const void*)k_motif<false, true> : (const void*)k_motif<false, false>);
-    GPM_CUDA(cudaFuncSetAttribute(kfun, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    allow_shared(kfun, smem);
     Grid gr = plan_grid(g, kfun, wpb, smem, max_per_sm);
     const long long nw = gr.total_warps();
     if (!smem_state) {
@@ -752,7 +752,7 @@ static void motif_count_noalloc(const int32_t* indptr, const int32_t* indices, i
     p.donate = 0;
     p.donate_min = 2;
     p.max_idle_ns = 120000000000ull;
-    GPM_CUDA(cudaFuncSetAttribute(k_motif<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    allow_shared((const void*)k_motif<true, false>, smem);
     int per_sm = 0;
     GPM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_motif<true, false>, wpb * 32, smem));
     if (per_sm <= 0) fail(GPM_EINVAL, "kernel cannot be resident");

@@ -491,7 +491,7 @@ Grid plan_hom(HomLaunch& p, int k, int sms) {
     gr.warps_per_block = HOM_WARPS;
     while (gr.warps_per_block > 1 && 4 * (size_t)p.warp_words * gr.warps_per_block > 220 * 1024) gr.warps_per_block /= 2;
     const size_t smem = 4 * (size_t)p.warp_words * gr.warps_per_block;
-    GPM_CUDA(cudaFuncSetAttribute(hom_kernel(k), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    allow_shared(hom_kernel(k), smem);
     const long long per_sm = std::max(1, resident_blocks(hom_kernel(k), gr.warps_per_block * 32, smem));
     // k = 5, few vertices: each is shared by several warps, so that the last
     // round of vertices is not a whole vertex long (block-model graph of 2,000

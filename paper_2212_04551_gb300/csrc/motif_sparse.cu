@@ -221,7 +221,7 @@ void run_motif_sparse(gpm_graph* g, int k, uint64_t* counts_out) {
         p.out = &r->hom[H_CYCLE4];
         if (smem) {
             const size_t bytes = sizeof(uint32_t) * (size_t)((g->n + 1) / 2);
-            GPM_CUDA(cudaFuncSetAttribute(k_cycle4<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+            allow_shared((const void*)k_cycle4<true>, bytes);
             k_cycle4<true><<<blocks, C4_THREADS, bytes, s>>>(p);
         } else {
             k_cycle4<false><<<blocks, C4_THREADS, 0, s>>>(p);

@@ -541,7 +541,7 @@ void mlp_grad(const uint16_t* w, const float* x, const float* t, int64_t n, floa
     GPM_CUDA(cudaGetDevice(&dev));
     GPM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const size_t smem = sizeof(float) * BW_SMEM;
-    GPM_CUDA(cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    allow_shared((const void*)k_mlp_backward, smem);
     const int blocks = (int)std::min<int64_t>((n + BW_TILE - 1) / BW_TILE, (int64_t)sms * 2);
     k_mlp_backward<<<blocks, BW_THREADS, smem, s>>>(w, x, t, n, grad, loss);
     GPM_CUDA(cudaGetLastError());

@@ -2,6 +2,8 @@
 of copies and launches, failing calls, limits.  CPU only."""
 from __future__ import annotations
 
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -72,3 +74,20 @@ def test_a_failed_first_batch_call_leaves_nothing_behind(gpu, kc, km):
         if not failed:
             break
     assert at > 3 and not failed
+
+
+@pytest.mark.parametrize("k", [5, 6])
+def test_a_smaller_graph_counted_meanwhile_takes_no_shared_memory_away(gpu, k):
+    """Between one call's plan and its launch, another (another thread's) counts
+    a small graph with the same kernel."""
+    n = {5: 9000, 6: 11000}[k]                              # more than 48 KB a block
+    big, small = gpu.graph(*_path(n)), gpu.graph(*_path(20))
+    seen = []
+    meanwhile = ctypes.CFUNCTYPE(None)(lambda: seen.append(gpu.motifs(small, k)))
+    gpu.log()
+    gpu.lib.fake_on_event_record(ctypes.cast(meanwhile, ctypes.c_void_p))
+    assert gpu.motifs(big, k) == gpm.GPM_OK, gpu.error()
+    assert seen == [gpm.GPM_OK]
+    assert max(x[3] for x in gpu.log()) > 48 * 1024
+    for g in (big, small):
+        gpu.lib.gpm_graph_destroy(g)
