@@ -74,8 +74,8 @@ struct gpm_batch {
             if (host_out) cudaFreeHost(host_out);
         }
     };
-    // (kc, km, wpb, bps, order, motif_agg_min, batch_split)
-    std::map<std::tuple<int, int, int, int, int, int, int>, Captured> graphs;
+    // (kc, km, motifs from homomorphism counts, wpb, bps, order, motif_agg_min, batch_split)
+    std::map<std::tuple<int, int, bool, int, int, int, int, int>, Captured> graphs;
 };
 
 namespace gpm {
@@ -313,15 +313,46 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     const int wpb = b->cfg.warps_per_block > 0 ? b->cfg.warps_per_block : 8;
     const int bps = b->cfg.blocks_per_sm;
     const int split = std::max(1, b->cfg.batch_split);
-    const auto key = std::make_tuple(kc, km, wpb, bps, b->order_mode, b->cfg.motif_agg_min, split);
-    auto it = b->graphs.find(key);
+    const int hom_k = km;
+    bool hom = km > 0 && b->cfg.motif_agg_min > 0 && hom_applies(b->max_graph_n, g->max_deg, km);
+    auto find = [&] {
+        return b->graphs.find({kc, hom_k, hom, wpb, bps, b->order_mode, b->cfg.motif_agg_min, split});
+    };
+    auto it = find();
     if (it != b->graphs.end()) return it->second;
 
     if (kc > 0) ensure_dag(g);
     DevBuf units, uranges;
     const int npat = km > 0 ? (int)pattern_table(km).num_patterns : 0;
-    const int hom_k = km;
-    const bool hom = km > 0 && b->cfg.motif_agg_min > 0 && hom_applies(b->max_graph_n, g->max_deg, km);
+    const size_t G = (size_t)b->n_graphs;
+    DevBuf dev_hom;
+    const size_t hom_bytes = sizeof(unsigned long long) * (G * HOM_N + 1);
+    HomLaunch hp{};
+    Grid hgr;
+    if (hom) try {
+        dev_hom.ensure(hom_bytes);
+        hp.indptr = g->indptr.as<int32_t>();
+        hp.indices = g->indices.as<int32_t>();
+        hp.deg = g->degree.as<int32_t>();
+        hp.goff = b->goff.as<int32_t>();
+        hp.vgraph = b->vgraph.as<int32_t>();
+        hp.n = g->n;
+        hp.grab = 16;     // neighbouring vertices: mostly one graph
+        hp.maxn = b->max_graph_n;
+        hp.maxd = std::max(g->max_deg, 1);
+        hp.hom = dev_hom.as<unsigned long long>();
+        hp.ticket = hp.hom + G * HOM_N;
+        if (hom_k == 5) hp.edges = ensure_hom_edges(g, hp.goff, hp.vgraph);
+        hgr = plan_hom(hp, hom_k, g->num_sms);
+        device_hom_table(hom_k, b->stream);
+    } catch (const Error& e) {
+        // the walk needs none of this; a later call tries again
+        if (e.status != GPM_ENOMEM) throw;
+        dev_hom.release();
+        hom = false;
+        it = find();
+        if (it != b->graphs.end()) return it->second;
+    }
     if (hom) km = 0;      // no motif units in k_batch
     const int hom_clique = hom && kc <= hom_k ? kc : 0;     // cliques from the motifs' sums
     const long long n_units = build_units(b, hom_clique ? 0 : kc, km, b->order_mode, split, units, uranges);
@@ -379,11 +410,9 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     gpm_batch::Captured c;
     c.units = std::move(units);
     c.uranges = std::move(uranges);
-    const size_t G = (size_t)b->n_graphs;
     const size_t ctl_words = (sizeof(Control) + 7) / 8;
     c.words = G + G * npat + ctl_words;
-    const size_t hom_bytes = sizeof(unsigned long long) * (G * HOM_N + 1);
-    if (hom) c.dev_hom.ensure(hom_bytes);
+    c.dev_hom = std::move(dev_hom);
     c.dev_out.ensure(sizeof(unsigned long long) * c.words);
     GPM_CUDA(cudaMallocHost(&c.host_out, sizeof(unsigned long long) * c.words));
     p.clique_out = c.dev_out.as<unsigned long long>();
@@ -392,28 +421,10 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     c.blocks = blocks;
     c.wpb = wpb;
     c.launches = (n_units > 0 ? 1 : 0) + (hom ? 2 : 0);
-    HomLaunch hp{};
-    Grid hgr;
-    if (hom) {
-        hp.indptr = p.indptr;
-        hp.indices = p.indices;
-        hp.deg = g->degree.as<int32_t>();
-        hp.goff = p.goff;
-        hp.vgraph = p.vgraph;
-        hp.n = g->n;
-        hp.grab = 16;     // neighbouring vertices: mostly one graph
-        hp.maxn = b->max_graph_n;
-        hp.maxd = std::max(g->max_deg, 1);
-        hp.hom = c.dev_hom.as<unsigned long long>();
-        hp.ticket = hp.hom + G * HOM_N;
-        hp.ctl = p.ctl;
-        if (hom_k == 5) hp.edges = ensure_hom_edges(g, hp.goff, hp.vgraph);
-        hgr = plan_hom(hp, hom_k, g->num_sms);
-        device_hom_table(hom_k, b->stream);
-        if (n_units == 0) {
-            c.blocks = hgr.blocks;
-            c.wpb = hgr.warps_per_block;
-        }
+    hp.ctl = p.ctl;
+    if (hom && n_units == 0) {
+        c.blocks = hgr.blocks;
+        c.wpb = hgr.warps_per_block;
     }
 
     cudaGraph_t graph = nullptr;
@@ -440,7 +451,8 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     cudaError_t e3 = cudaGraphInstantiate(&c.exec, graph, 0);
     cudaGraphDestroy(graph);
     check_cuda(e3, "cudaGraphInstantiate");
-    return b->graphs.emplace(key, std::move(c)).first->second;
+    return b->graphs.emplace(std::make_tuple(kc, hom_k, hom, wpb, bps, b->order_mode, b->cfg.motif_agg_min, split),
+                             std::move(c)).first->second;
 }
 
 // One replay; results in cap.host_out.  Returns the device time (ms).

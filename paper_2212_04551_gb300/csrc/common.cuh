@@ -171,6 +171,7 @@ struct Grid {
 
 // graph.cu
 void ensure_dag(gpm_graph* g);
+void release_dag(gpm_graph* g);   // the orientation and the root order built on it; max_outdeg stays known
 const int32_t* ensure_root_order(gpm_graph* g, int app);  // plain scheduler order
 const int32_t* ensure_id_order(gpm_graph* g);             // 0, 1, ..., n-1
 long long roots_at_least(gpm_graph* g, int d);            // vertices of out-degree >= d: the first ones of the clique order

@@ -397,6 +397,11 @@ void ensure_dag(gpm_graph* g) {
     g->dag_ready = true;
 }
 
+void release_dag(gpm_graph* g) {
+    g->dag_ready = g->order_clique_ready = false;
+    for (DevBuf* b : {&g->dag_off, &g->dag_adj, &g->dag_outdeg, &g->order_clique}) b->release();
+}
+
 const int32_t* ensure_root_order(gpm_graph* g, int app) {
     if (app == GPM_APP_CLIQUE) {
         ensure_dag(g);

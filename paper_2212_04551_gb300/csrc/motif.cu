@@ -311,6 +311,28 @@ __global__ void k_motif_seed(const int32_t* __restrict__ roots, long long n_coun
     }
 }
 
+// Counts from homomorphism counts (motif_hom.cu, motif_sparse.cu), where these
+// apply and their scratch fits: with little memory left (the orientation and a
+// counter per edge can take more than the walk's marks) the walk still counts.
+static bool motif_from_sums(gpm_graph* g, int k, uint64_t* counts_out) {
+    const bool had_dag = g->dag_ready;
+    try {
+        if (hom_applies(g->n, g->max_deg, k) && (k == 5 || g->max_deg <= (k == 3 ? HOM_HUB_D3 : HOM_HUB_D4))) {
+            run_motif_hom(g, k, counts_out);
+            return true;
+        }
+        if (motif_sparse_applies(g, k)) {
+            run_motif_sparse(g, k, counts_out);
+            return true;
+        }
+    } catch (const Error& e) {
+        if (e.status != GPM_ENOMEM) throw;
+        g->scratch_slab.release();
+        if (!had_dag) release_dag(g);
+    }
+    return false;
+}
+
 void run_motif(gpm_graph* g, int k, const int32_t* d_roots, int64_t n_roots,
                unsigned long long* d_per_root, uint64_t* counts_out, int64_t n_counter, const SplitPlan* plan,
                double monitor_threshold, MonitorStats* monitor_stats, ListJob* list) {
@@ -321,19 +343,12 @@ void run_motif(gpm_graph* g, int k, const int32_t* d_roots, int64_t n_roots,
     const PatternTable& tab = pattern_table(k);
     const int npat = (int)tab.num_patterns;
     cudaStream_t s = g->stream;
-    // Whole-graph counts of small patterns come from homomorphism counts
-    // (motif_hom.cu, motif_sparse.cu); lists of roots, schedules, per-root results, listing and
-    // monitored runs are defined on the walk, and so is motif_agg_min = 0.
-    if (!d_roots && !plan && !d_per_root && !monitored && !list && g->cfg.motif_agg_min > 0) {
-        if (hom_applies(g->n, g->max_deg, k) && (k == 5 || g->max_deg <= (k == 3 ? HOM_HUB_D3 : HOM_HUB_D4))) {
-            run_motif_hom(g, k, counts_out);
-            return;
-        }
-        if (motif_sparse_applies(g, k)) {
-            run_motif_sparse(g, k, counts_out);
-            return;
-        }
-    }
+    // Whole-graph counts of small patterns come from homomorphism counts; lists
+    // of roots, schedules, per-root results, listing and monitored runs are
+    // defined on the walk, and so is motif_agg_min = 0.
+    if (!d_roots && !plan && !d_per_root && !monitored && !list && g->cfg.motif_agg_min > 0 &&
+        motif_from_sums(g, k, counts_out))
+        return;
     if (!d_roots) {
         d_roots = ensure_root_order(g, GPM_APP_MOTIF);
         n_roots = g->n;

@@ -170,8 +170,14 @@ bool motif_sparse_applies(gpm_graph* g, int k) {
     double bound = (double)g->nnz;
     for (int i = 2; i < k; i++) bound *= (double)std::max(g->max_deg, 1);
     if (bound >= 9.0e18 || g->max_deg >= 65536) return false;   // (16-bit counters)
+    // (int32 offsets of the padded orientation)
+    if (g->nnz / 2 + 3 * std::min<long long>(g->n, g->nnz / 2) >= INT32_MAX) return false;
+    if (g->max_outdeg > 1024) return false;                     // no list path
+    const bool built = g->dag_ready;
     ensure_dag(g);
-    return g->max_outdeg <= 1024;                               // no list path
+    if (g->max_outdeg <= 1024) return true;
+    if (!built) release_dag(g);                                 // the walk does not use it
+    return false;
 }
 
 void run_motif_sparse(gpm_graph* g, int k, uint64_t* counts_out) {

@@ -58,7 +58,9 @@ def test_a_failed_first_batch_call_leaves_nothing_behind(gpu, kc, km):
     """Whatever allocation (or step of the capture) fails in a batch's first
     call, the next one tries again and succeeds, and nothing is leaked."""
     warm = gpu.batch(*_two_paths(20))                       # the tables of the process
-    assert gpu.batch_count(warm, kc, km, 2) == gpm.GPM_OK, gpu.error()
+    for agg in (16, 0):
+        gpu.configure(warm, batch=True, motif_agg_min=agg)
+        assert gpu.batch_count(warm, kc, km, 2) == gpm.GPM_OK, gpu.error()
     gpu.lib.gpm_batch_destroy(warm)
     before = gpu.lib.fake_memory_in_use()
     for at in range(1, 100):
@@ -66,7 +68,8 @@ def test_a_failed_first_batch_call_leaves_nothing_behind(gpu, kc, km):
         gpu.lib.fake_fail(b"alloc", at)
         st = gpu.batch_count(b, kc, km, 2)
         failed = gpu.lib.fake_failed()
-        assert st == (gpm.GPM_ENOMEM if failed else gpm.GPM_OK), (at, gpu.error())
+        # (what only the homomorphism counts need is not missed: the walk counts)
+        assert st == gpm.GPM_OK or (failed and st == gpm.GPM_ENOMEM), (at, gpu.error())
         gpu.lib.fake_fail(b"", 0)
         assert gpu.batch_count(b, kc, km, 2) == gpm.GPM_OK, (at, gpu.error())
         gpu.lib.gpm_batch_destroy(b)
@@ -91,3 +94,36 @@ def test_a_smaller_graph_counted_meanwhile_takes_no_shared_memory_away(gpu, k):
     assert max(x[3] for x in gpu.log()) > 48 * 1024
     for g in (big, small):
         gpu.lib.gpm_graph_destroy(g)
+
+
+@pytest.mark.parametrize("n,k", [(300, 3), (300, 5), (20000, 3), (20000, 4), (200000, 4)])
+def test_motifs_are_counted_without_the_memory_for_the_homomorphism_sums(gpu, n, k):
+    """Whichever allocation of the sums' route fails, the walk counts, and what
+    the attempt took is given back."""
+    warm = gpu.graph(*_path(n))
+    for agg in (16, 0):
+        gpu.configure(warm, motif_agg_min=agg)
+        assert gpu.motifs(warm, k) == gpm.GPM_OK, gpu.error()
+    gpu.lib.gpm_graph_destroy(warm)
+    walk = gpu.graph(*_path(n))
+    gpu.configure(walk, motif_agg_min=0)
+    before = gpu.lib.fake_memory_in_use()
+    assert gpu.motifs(walk, k) == gpm.GPM_OK, gpu.error()
+    walked = gpu.lib.fake_memory_in_use() - before
+    gpu.lib.gpm_graph_destroy(walk)
+    for at in range(1, 100):
+        g = gpu.graph(*_path(n))
+        before = gpu.lib.fake_memory_in_use()
+        gpu.log()
+        gpu.lib.fake_fail(b"cudaMalloc", at)
+        assert gpu.motifs(g, k) == gpm.GPM_OK, (at, gpu.error())
+        failed = gpu.lib.fake_failed()
+        gpu.lib.fake_fail(b"", 0)
+        assert failed == any("k_motif" in x[0] for x in gpu.log())
+        if failed:
+            # (besides the walk's: small scratch only)
+            assert gpu.lib.fake_memory_in_use() - before <= walked + 4 * n + 4096
+        gpu.lib.gpm_graph_destroy(g)
+        if not failed:
+            break
+    assert at > 1 and not failed
