@@ -54,7 +54,7 @@ constexpr int NE_LIGHT_GRAB = 8;      // roots a warp takes at a time
 constexpr int NE_WARPS = 4;           // warps per block of the heavy launch
 constexpr int NE_HELP_D = 128;        // roots above this are offered to further blocks ...
 constexpr int NE_HELP_ROUNDS = 24;    // ... this many times (k >= 6, where a child's work can be large)
-constexpr int NE_SCRATCH = 64 + 128;   // words for a second re-indexing (ne_quads_small)
+constexpr int NE_SCRATCH = 64 + 128;   // words for a second re-indexing (ne_four_again)
 constexpr int NE_FILTER_WORDS = 64;   // hash filter of N+(r): 2,048 bits
 
 struct NeLaunch {
@@ -390,7 +390,10 @@ __device__ __forceinline__ void ne_child(const NeLaunch& p, NeCount& c, const Ne
         if (load) lv = h;
 #pragma unroll 1
         for (;;) {
-            if (todo == NE_INDEX) ne_indexed(p, c, k, rows, m, a, h, lane);
+            if (todo == NE_INDEX) {
+                ne_indexed(p, c, k, rows, m, a, h, lane);
+                if (lv >= 2) ne_settle(p.ne, c, lane);
+            }
             if (over) {        // nothing is left of the wide set
                 lv--;
                 load = true;

@@ -52,9 +52,10 @@ constexpr int NE_SPARSE = 16;
 // size k_hi - q in acc[q] (24 makes every lane's share a whole number; a
 // lane's sum may be negative, the warp's is not).  A set adds less than 2^41
 // to acc[0] (members^4), less to the others; all are folded into `size` (with
-// carry checks) before acc[0] or acc[1] passes 2^58 and at the end of a root
-// (heavy launch) or of the warp (light launch: 32 members at most), so that none
-// can wrap.
+// carry checks) at the end of a root (heavy launch) or of the warp (light
+// launch: 32 members at most).  Where a root can have any number of sets --
+// four sizes to go, or below a wide set -- ne_settle folds after a set that
+// brought acc[0] or acc[1] past 2^57, so that none can wrap.
 struct NeCount {
     unsigned long long size = 0;     // lane s: cliques of size s
     long long acc[5] = {0, 0, 0, 0, 0};
@@ -112,6 +113,12 @@ __device__ __forceinline__ void ne_fold(const NeParams& p, NeCount& c, int lane)
         c.acc[q] = 0;
     }
     c.size = gpm_add_cc(c.size, v, c.ovf);
+}
+
+// The same once a sum has passed 2^57, between two sets (all lanes must call).
+__device__ __forceinline__ void ne_settle(const NeParams& p, NeCount& c, int lane) {
+    const bool full = ((unsigned long long)(c.acc[0] + (1ll << 57)) | (unsigned long long)(c.acc[1] + (1ll << 57))) >> 58;
+    if (__any_sync(GPM_FULL_MASK, full)) ne_fold(p, c, lane);
 }
 
 // The non-edges of the lane's members of S (members 32 x + lane).
@@ -484,8 +491,7 @@ __device__ __forceinline__ void ne_sets(const NeParams& p, NeCount& c, int m, in
                     else if (m4 <= 64) ne_four_again<W, 2>(p, c, some, m4, a + s - m4, Hs, scratch, scratch + 64, lane);
                 }
             }
-            const bool full = ((unsigned long long)(c.acc[0] + (1ll << 57)) | (unsigned long long)(c.acc[1] + (1ll << 57))) >> 58;
-            if (__any_sync(GPM_FULL_MASK, full)) ne_fold(p, c, lane);
+            ne_settle(p, c, lane);
         }
         if (!four) {
             c.wops += (unsigned)(s * W);
