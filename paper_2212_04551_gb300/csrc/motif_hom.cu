@@ -342,7 +342,8 @@ __device__ __forceinline__ void hom_vertex(const HomLaunch& p, const HomWarp& k,
                     for (; q < e; q += 8) {
                         const int x = p.indices[q] - base;
                         if (x >= hi) break;
-                        atomicOr(&k.M[(x - lo) * w + (i >> 5)], 1u << (i & 31));
+                        // (an unchecked graph's lists may not be sorted)
+                        if (x >= lo) atomicOr(&k.M[(x - lo) * w + (i >> 5)], 1u << (i & 31));
                         done++;
                     }
                     if (i < d && done) atomicAdd(&k.at[i], done);

@@ -82,8 +82,9 @@ static void simt_entry() {
 
 // fn by one block of `threads` threads with `words` words of shared memory
 static void simt_run(int threads, size_t words, std::function<void()> fn) {
-    std::vector<uint32_t> smem(words + 72, 0xdeadbeefu);
-    simt_smem = smem.data() + 32;
+    const size_t guard = 1 << 14;      // words watched on either side
+    std::vector<uint32_t> smem(words + 2 * guard, 0xdeadbeefu);
+    simt_smem = smem.data() + guard;
     S.fn = fn;
     S.threads = threads;
     S.f.clear();
@@ -127,7 +128,7 @@ static void simt_run(int threads, size_t words, std::function<void()> fn) {
         }
     }
     for (size_t i = 0; i < smem.size(); i++)
-        if ((i < 32 || i >= words + 32) && smem[i] != 0xdeadbeefu) {
+        if ((i < guard || i >= words + guard) && smem[i] != 0xdeadbeefu) {
             fprintf(stderr, "write outside of shared memory\n");
             abort();
         }

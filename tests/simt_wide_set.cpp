@@ -1,9 +1,10 @@
 // The sets of one root's child (ne_child, clique_nonedge.cu) on the CPU: a
 // candidate set of 66 disjoint non-edges and three hubs, each non-adjacent to
 // half of the others.  The hubs are taken out one by one, the set that holds
-// each has three sizes to go, and what is left is counted as a matching.  argv: what every lane holds in acc[0] from the root's earlier
-// sets.  Prints the largest |acc[0]| over the lanes afterwards, and the cliques
-// counted once all is folded.
+// each has three sizes to go, and what is left is counted as a matching.
+// argv[1]: what every lane holds in acc[0] from the root's earlier sets.  Prints
+// the largest |acc[0]| over the lanes afterwards, the cliques counted once all
+// is folded, and the set's 4-cliques.
 #include "simt.h"
 #include "device_part.h"
 
