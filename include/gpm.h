@@ -94,9 +94,9 @@ gpm_status gpm_graph_info(const gpm_graph* g, int32_t* n, int64_t* m, int32_t* m
  * lowest-(degree, id) vertex), which plays the role of the paper's "lower"
  * filter.  Roots with at most 1,024 out-neighbours are counted on bitmaps of
  * their out-neighbourhood in shared memory, branching on the non-edges of the
- * candidate sets (clique_cpl = 0, a chosen clique_tail or clique_compact, or a
- * root order other than the default: by walking the cliques instead); roots
- * above that, in the same call, by sorted-list intersection (the paper's
+ * candidate sets (with a clique_tail, clique_compact, clique_compact3 or
+ * clique_cpl other than the default, which choose among the tails of the walk,
+ * or another root order: by walking the cliques instead); roots above that, in the same call, by sorted-list intersection (the paper's
  * extension arrays) with per-warp lists in device memory.  out_count: host pointer to one uint64.
  * Errors: GPM_EINVAL, GPM_ENOMEM, GPM_ECUDA, GPM_ETIMEOUT, GPM_EOVERFLOW.
  */
@@ -195,8 +195,7 @@ typedef struct {
                                /* sum_t C(a_t, 2) minus the open wedges found from the non-edges,     */
                                /* instead of one AND + POPC per (k-1)-clique: 0 never, 1 always,      */
                                /* 2..100 for tail nodes whose members are at least this percent       */
-                               /* pairwise adjacent (default 85); 0 also makes whole-graph counts     */
-                               /* walk the cliques                                                    */
+                               /* pairwise adjacent (default 85)                                      */
 } gpm_config;
 
 #define GPM_ORDER_ID          0  /* roots in id order                               */

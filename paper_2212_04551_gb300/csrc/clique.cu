@@ -392,8 +392,10 @@ void run_clique(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_
     // walking the cliques.  Root lists, schedules and per-root results keep
     // the walk below, whose units, hand-offs and bounded waits they are
     // defined on, and so does a caller that chooses one of the walk's tails.
-    const bool nonedge = whole && !d_per_root && k_hi >= 3 && g->cfg.clique_cpl != 0 && g->cfg.clique_tail == 0 &&
-                         g->cfg.clique_compact == 0;
+    const gpm_config def = default_config();
+    const bool nonedge = whole && !d_per_root && k_hi >= 3 && g->cfg.clique_cpl == def.clique_cpl &&
+                         g->cfg.clique_tail == def.clique_tail && g->cfg.clique_compact == def.clique_compact &&
+                         g->cfg.clique_compact3 == def.clique_compact3;
     if (n_counter < 0 || n_counter > n_roots) n_counter = n_roots;
     const int n_split = (int)(n_roots - n_counter);
     const int split_chunks = plan ? plan->chunks : 0;

@@ -127,3 +127,15 @@ def test_motifs_are_counted_without_the_memory_for_the_homomorphism_sums(gpu, n,
         if not failed:
             break
     assert at > 1 and not failed
+
+
+@pytest.mark.parametrize("tail", [dict(clique_cpl=0), dict(clique_cpl=1), dict(clique_cpl=50), dict(clique_tail=2),
+                                  dict(clique_tail=3), dict(clique_compact=1), dict(clique_compact=2),
+                                  dict(clique_compact3=0), dict(clique_compact3=2), {}])
+def test_a_chosen_tail_of_the_clique_walk_is_walked(gpu, tail):
+    g = gpu.graph(*_path(30))
+    gpu.configure(g, **tail)
+    gpu.log()
+    assert gpu.cliques(g, 7) == gpm.GPM_OK and gpu.cliques(g, 4, 8) == gpm.GPM_OK, gpu.error()
+    assert sum("8k_cliqueE" in x[0] for x in gpu.log()) == (2 if tail else 0)
+    gpu.lib.gpm_graph_destroy(g)
