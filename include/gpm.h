@@ -168,8 +168,10 @@ typedef struct {
     int32_t warps_per_block;   /* 1, 2, 4, 8 or 16 (0 = automatic: the most resident   */
                                /* warps per SM for cliques; 4 for motifs, whose grid, */
                                /* when the marks live in HBM, is sized so that every  */
-                               /* warp's marks fit in L2)                              */
-    int32_t blocks_per_sm;     /* resident blocks per SM (0 = automatic)               */
+                               /* warp's marks fit in L2).  The homomorphism counts    */
+                               /* use at most 4; whole-graph clique counts and the    */
+                               /* edge sums have blocks of a fixed size               */
+    int32_t blocks_per_sm;     /* resident blocks per SM, at most (0 = automatic)      */
     int32_t donate_min;        /* split a level only if >= this many siblings remain  */
     int32_t order;             /* GPM_ORDER_* root order of the plain scheduler         */
     int32_t max_idle_ms;       /* bounded wait: an idle warp gives up after this long  */

@@ -343,7 +343,7 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
         hp.hom = dev_hom.as<unsigned long long>();
         hp.ticket = hp.hom + G * HOM_N;
         if (hom_k == 5) hp.edges = ensure_hom_edges(g, hp.goff, hp.vgraph);
-        hgr = plan_hom(hp, hom_k, g->num_sms);
+        hgr = plan_hom(hp, hom_k, g->num_sms, b->cfg);
         device_hom_table(hom_k, b->stream);
     } catch (const Error& e) {
         // the walk needs none of this; a later call tries again

@@ -648,15 +648,12 @@ int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* 
         p.first = big;
         p.last = all;
         p.ticket = tickets + 16;
-        const int per_sm = resident_blocks((const void*)k_clique_ne_light, NE_LIGHT_WARPS * 32, 0);
         const long long want = (all - big + NE_LIGHT_GRAB * NE_LIGHT_WARPS - 1) / (NE_LIGHT_GRAB * NE_LIGHT_WARPS);
-        const int blocks = (int)std::min<long long>(want, (long long)per_sm * g->num_sms);
-        k_clique_ne_light<<<blocks, NE_LIGHT_WARPS * 32, 0, s>>>(p);
+        Grid gr = plan_grid(g, (const void*)k_clique_ne_light, NE_LIGHT_WARPS, 0);
+        gr.blocks = (int)std::min<long long>(want, gr.blocks);
+        k_clique_ne_light<<<gr.blocks, NE_LIGHT_WARPS * 32, 0, s>>>(p);
         GPM_CUDA(cudaGetLastError());
-        if (!launches) {
-            grid->blocks = blocks;
-            grid->warps_per_block = NE_LIGHT_WARPS;
-        }
+        if (!launches) *grid = gr;
         launches++;
     }
     return launches;

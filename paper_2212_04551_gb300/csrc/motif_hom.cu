@@ -485,15 +485,16 @@ const uint32_t* ensure_hom_edges(gpm_graph* g, const int32_t* goff, const int32_
     return g->hom_edges.as<uint32_t>();
 }
 
-Grid plan_hom(HomLaunch& p, int k, int sms) {
+Grid plan_hom(HomLaunch& p, int k, int sms, const gpm_config& cfg) {
     p.warp_words = hom_warp_words(p.maxn, p.maxd, k);
     p.m_words = hom_m_words(p.maxn, p.maxd);
     Grid gr;
-    gr.warps_per_block = HOM_WARPS;
+    gr.warps_per_block = cfg.warps_per_block > 0 ? std::min(cfg.warps_per_block, HOM_WARPS) : HOM_WARPS;
     while (gr.warps_per_block > 1 && 4 * (size_t)p.warp_words * gr.warps_per_block > 220 * 1024) gr.warps_per_block /= 2;
     const size_t smem = 4 * (size_t)p.warp_words * gr.warps_per_block;
     allow_shared(hom_kernel(k), smem);
-    const long long per_sm = std::max(1, resident_blocks(hom_kernel(k), gr.warps_per_block * 32, smem));
+    long long per_sm = std::max(1, resident_blocks(hom_kernel(k), gr.warps_per_block * 32, smem));
+    if (cfg.blocks_per_sm > 0) per_sm = std::min<long long>(per_sm, cfg.blocks_per_sm);
     // k = 5, few vertices: each is shared by several warps, so that the last
     // round of vertices is not a whole vertex long (block-model graph of 2,000
     // vertices on 1,824 warps)
@@ -532,7 +533,7 @@ void run_motif_hom(gpm_graph* g, int k, uint64_t* counts_out) {
     p.ticket = &r->ctl.next_root;
     p.ctl = &r->ctl;
     if (k == 5) p.edges = ensure_hom_edges(g, nullptr, nullptr);
-    const Grid gr = plan_hom(p, k, g->num_sms);
+    const Grid gr = plan_hom(p, k, g->num_sms, g->cfg);
     GPM_CUDA(cudaEventRecord(g->ev0, s));
     GPM_CUDA(launch_hom(p, k, gr, s));
     GPM_CUDA(cudaEventRecord(g->ev1, s));

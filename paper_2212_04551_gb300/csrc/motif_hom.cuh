@@ -65,7 +65,7 @@ int hom_m_words(int n, int d);
 const uint32_t* ensure_hom_edges(gpm_graph* g, const int32_t* goff, const int32_t* vgraph);
 // Fills warp_words and sizes the launch (no stream operations); the launch itself (nothing
 // throws between the two ends of a capture).
-Grid plan_hom(HomLaunch& p, int k, int sms);
+Grid plan_hom(HomLaunch& p, int k, int sms, const gpm_config& cfg);
 cudaError_t launch_hom(const HomLaunch& p, int k, const Grid& gr, cudaStream_t s);
 // Whole-graph counts of g where hom_applies (stats filled)
 void run_motif_hom(gpm_graph* g, int k, uint64_t* counts_out);

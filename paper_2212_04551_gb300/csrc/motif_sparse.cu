@@ -209,7 +209,8 @@ void run_motif_sparse(gpm_graph* g, int k, uint64_t* counts_out) {
     Grid gr;
     GPM_CUDA(cudaEventRecord(g->ev0, s));
     int launches = launch_clique_nonedge(g, 3, k, &r->ctl, &gr, tri);
-    k_edge_sums<<<std::max(1, std::min((g->n + 31) / 32, g->num_sms * 8)), 256, 0, s>>>(
+    const int per_sm = g->cfg.blocks_per_sm > 0 ? std::min(g->cfg.blocks_per_sm, 8) : 8;
+    k_edge_sums<<<std::max(1, std::min((g->n + 31) / 32, g->num_sms * per_sm)), 256, 0, s>>>(
         g->dag_off.as<int32_t>(), g->dag_adj.as<int32_t>(), g->dag_outdeg.as<int32_t>(), g->degree.as<int32_t>(), tri,
         g->n, r->hom);
     GPM_CUDA(cudaGetLastError());

@@ -139,3 +139,28 @@ def test_a_chosen_tail_of_the_clique_walk_is_walked(gpu, tail):
     assert gpu.cliques(g, 7) == gpm.GPM_OK and gpu.cliques(g, 4, 8) == gpm.GPM_OK, gpu.error()
     assert sum("8k_cliqueE" in x[0] for x in gpu.log()) == (2 if tail else 0)
     gpu.lib.gpm_graph_destroy(g)
+
+
+@pytest.mark.parametrize("n,k,kernel", [(9000, 5, "5k_homILi5"), (400, 4, "5k_homILi4"), (200000, 3, "11k_edge_sums"),
+                                        (9000, 6, "7k_motif")])
+def test_launch_shapes_follow_the_configuration(gpu, n, k, kernel):
+    """blocks_per_sm bounds every launch over the vertices; warps_per_block is
+    the kernel's, where it has a choice."""
+    g = gpu.graph(*_path(n))
+    for wpb, bps in ((0, 0), (0, 1), (1, 1), (2, 1), (16, 2)):
+        gpu.configure(g, warps_per_block=wpb, blocks_per_sm=bps)
+        gpu.log()
+        assert gpu.motifs(g, k) == gpm.GPM_OK, gpu.error()
+        (_, blocks, threads, _), = [x for x in gpu.log() if kernel in x[0]]
+        assert blocks <= 152 * (bps or 32)
+        if "k_hom" in kernel:
+            assert threads <= 128 and (not wpb or threads <= 32 * wpb)
+    gpu.lib.gpm_graph_destroy(g)
+    b = gpu.batch(*_two_paths(2000))
+    for wpb, bps in ((1, 1), (2, 2), (16, 1)):
+        gpu.configure(b, batch=True, warps_per_block=wpb, blocks_per_sm=bps)
+        gpu.log()
+        assert gpu.batch_count(b, 0, 5, 2) == gpm.GPM_OK, gpu.error()
+        (_, blocks, threads, _), = [x for x in gpu.log() if "k_homILi5" in x[0]]
+        assert blocks <= 152 * bps and threads <= 32 * wpb
+    gpu.lib.gpm_batch_destroy(b)
