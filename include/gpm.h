@@ -220,7 +220,10 @@ typedef struct {
     int32_t  kernel_launches;  /* kernels the call launched (enumeration path)    */
     uint64_t busy_warp_ns;     /* sum over the grid's warps of the time spent      */
                                /* inside work units (%globaltimer); 1 - busy /     */
-                               /* (warps x kernel time) is the idle warp fraction  */
+                               /* (warps x kernel time) is the idle warp fraction. */
+                               /* Of several launches: grid_blocks and             */
+                               /* warps_per_block are the first one's, and each    */
+                               /* launch's time is scaled to that grid             */
 } gpm_stats;
 
 gpm_status gpm_get_stats(const gpm_graph* g, gpm_stats* out);

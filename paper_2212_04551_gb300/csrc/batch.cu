@@ -63,12 +63,13 @@ struct gpm_batch {
         gpm::DevBuf dev_hom;         // [G][HOM_N] homomorphism sums, then the launch's ticket
         unsigned long long* host_out = nullptr;   // pinned
         size_t words = 0;
-        int blocks = 0, wpb = 0, launches = 0;
+        gpm::Launches made;          // k_batch and k_hom, where launched
+        int launches = 0;
         Captured() = default;
         Captured(Captured&& o) noexcept
             : exec(std::exchange(o.exec, nullptr)), units(std::move(o.units)), uranges(std::move(o.uranges)),
               dev_out(std::move(o.dev_out)), dev_hom(std::move(o.dev_hom)), host_out(std::exchange(o.host_out, nullptr)),
-              words(o.words), blocks(o.blocks), wpb(o.wpb), launches(o.launches) {}
+              words(o.words), made(o.made), launches(o.launches) {}
         ~Captured() {
             if (exec) cudaGraphExecDestroy(exec);
             if (host_out) cudaFreeHost(host_out);
@@ -418,14 +419,10 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     p.clique_out = c.dev_out.as<unsigned long long>();
     p.motif_out = p.clique_out + G;
     p.ctl = reinterpret_cast<Control*>(p.motif_out + G * npat);
-    c.blocks = blocks;
-    c.wpb = wpb;
+    if (n_units > 0 || !hom) c.made.add(p.ctl, Grid{blocks, wpb});
     c.launches = (n_units > 0 ? 1 : 0) + (hom ? 2 : 0);
     hp.ctl = p.ctl;
-    if (hom && n_units == 0) {
-        c.blocks = hgr.blocks;
-        c.wpb = hgr.warps_per_block;
-    }
+    if (hom) hp.busy = c.made.add(p.ctl, hgr);
 
     cudaGraph_t graph = nullptr;
     GPM_CUDA(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
@@ -571,10 +568,10 @@ void batch_count(gpm_batch* b, int kc, int km, uint64_t* clique_counts, uint64_t
     gpm_stats st{};
     st.kernel_ms = ms;
     st.units_done = h->units_done;
-    st.busy_warp_ns = h->busy_ns;
+    st.busy_warp_ns = cap.made.busy_ns(*h);
     st.kernel_launches = cap.launches;
-    st.grid_blocks = cap.blocks;
-    st.warps_per_block = cap.wpb;
+    st.grid_blocks = cap.made.grid[0].blocks;
+    st.warps_per_block = cap.made.grid[0].warps_per_block;
     b->stats = st;
     if (h->error == DEV_EINVAL) fail(GPM_ECUDA, "pattern table lookup hit an invalid traversal code");
     if (h->error >= DEV_ECHECK) fail(GPM_ECUDA, "device consistency check " + std::to_string(h->error - DEV_ECHECK) + " failed");

@@ -413,6 +413,7 @@ void run_clique(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_
         GPM_CUDA(cudaMemsetAsync(d_per_root, 0, sizeof(unsigned long long) * n_roots, s));
 
     gpm_stats st{};
+    Launches made;         // of the branching on non-edges
     int launches = 0;
     bool timed = false;
     if (k_hi <= 2) {
@@ -424,14 +425,14 @@ void run_clique(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_
             GPM_CUDA(cudaGetLastError());
         }
     } else if (n_roots > 0 && nonedge) {
-        Grid gr;
         GPM_CUDA(cudaEventRecord(g->ev0, s));
-        launches = launch_clique_nonedge(g, k_lo, k_hi, ctl, &gr);
+        launch_clique_nonedge(g, k_lo, k_hi, ctl, made);
         run_clique_list(g, k_lo, k_hi, d_roots, n_roots, d_per_root, ctl, CQ_MAX_OUTDEG);
         GPM_CUDA(cudaEventRecord(g->ev1, s));
         timed = true;
-        st.grid_blocks = gr.blocks;
-        st.warps_per_block = gr.warps_per_block;
+        launches = made.n;
+        st.grid_blocks = made.grid[0].blocks;
+        st.warps_per_block = made.grid[0].warps_per_block;
     } else if (n_roots > 0) {
         CliqueLaunch L = plan_clique_launch(g, k_lo, k_hi, d_roots, n_counter, n_seed, 0);
         CliqueParams& p = L.p;
@@ -461,7 +462,7 @@ void run_clique(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_
     st.donations = h.donations;
     st.idle_polls = h.idle_polls;
     st.word_ops = h.word_ops;
-    st.busy_warp_ns = h.busy_ns;
+    st.busy_warp_ns = made.busy_ns(h);
     st.kernel_launches = k_hi <= 2 && n_roots > 0 ? 1 : launches;
     if (timed && g->max_outdeg > CQ_MAX_OUTDEG) st.kernel_launches += 2;   // the list path
     g->stats = st;

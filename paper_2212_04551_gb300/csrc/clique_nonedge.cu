@@ -73,6 +73,7 @@ struct NeLaunch {
     unsigned int* tri;                    // nullable: triangles per out-list entry (rounds = 0)
     NeParams ne;
     Control* ctl;
+    unsigned long long* busy;             // this launch's warp time
     unsigned long long* ticket;           // next position (light) or root offer (heavy)
 };
 
@@ -80,8 +81,10 @@ __device__ __forceinline__ unsigned ne_hash(int x) { return (unsigned)x * 265443
 
 // End of a block: its warps' counts are added up in shared memory first (one
 // global add per size and block; thousands of warps would queue on each).
-__device__ __forceinline__ void ne_finish(const NeParams& ne, NeCount& c, Control* ctl, unsigned long long units,
+__device__ __forceinline__ void ne_finish(const NeLaunch& p, NeCount& c, unsigned long long units,
                                           unsigned long long busy, int lane) {
+    const NeParams& ne = p.ne;
+    Control* ctl = p.ctl;
     __shared__ unsigned long long sum[NE_LEVELS + 3];
     ne_fold(ne, c, lane);
     if (threadIdx.x < NE_LEVELS + 3) sum[threadIdx.x] = 0ull;
@@ -97,7 +100,7 @@ __device__ __forceinline__ void ne_finish(const NeParams& ne, NeCount& c, Contro
     const int t = threadIdx.x;
     if (t < NE_LEVELS) gpm_atomic_add_cc(&ctl->counts[t], sum[t], &ctl->overflow);
     else if (t < NE_LEVELS + 3 && sum[t])
-        atomicAdd(t == NE_LEVELS ? &ctl->units_done : t == NE_LEVELS + 1 ? &ctl->word_ops : &ctl->busy_ns, sum[t]);
+        atomicAdd(t == NE_LEVELS ? &ctl->units_done : t == NE_LEVELS + 1 ? &ctl->word_ops : p.busy, sum[t]);
 }
 
 // ------------------------------------------------------------------- light
@@ -196,7 +199,7 @@ __global__ void __launch_bounds__(NE_LIGHT_WARPS * 32) k_clique_ne_light(NeLaunc
         units += (unsigned)nr;
     }
     busy = gpm_globaltimer() - t0;
-    ne_finish(p.ne, c, p.ctl, units, busy, lane);
+    ne_finish(p, c, units, busy, lane);
 }
 
 // ------------------------------------------------------------------- heavy
@@ -565,7 +568,7 @@ __global__ void __launch_bounds__(NE_WARPS * 32, DEEP ? 5 : 10) k_clique_ne_heav
         if (threadIdx.x == 0) units++;
         busy += gpm_globaltimer() - t_unit;
     }
-    ne_finish(p.ne, c, p.ctl, units, busy, lane);
+    ne_finish(p, c, units, busy, lane);
 }
 
 // ------------------------------------------------------------------- host
@@ -595,9 +598,8 @@ static const unsigned long long* device_binomials(cudaStream_t s) {
 }
 
 // Whole-graph clique counts of sizes k_lo .. k_hi (k_hi >= 3) into ctl (its
-// counters zero); roots above the bitmap limit are left out.  Returns the
-// number of launches; grid/warps of the larger one for the statistics.
-int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* grid, unsigned int* tri) {
+// counters zero); roots above the bitmap limit are left out.
+void launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Launches& made, unsigned int* tri) {
     cudaStream_t s = g->stream;
     NeLaunch p{};
     p.roots = ensure_root_order(g, GPM_APP_CLIQUE);
@@ -619,7 +621,6 @@ int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* 
     g->scratch_queue.ensure(256 + sizeof(unsigned int) * (size_t)std::max<long long>(n_big, 1));
     unsigned long long* tickets = g->scratch_queue.as<unsigned long long>();
     GPM_CUDA(cudaMemsetAsync(tickets, 0, 256 + sizeof(unsigned int) * (size_t)n_big, s));
-    int launches = 0;
     if (n_big > 0) {
         p.first = above;
         p.last = big;
@@ -638,11 +639,10 @@ int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* 
         allow_shared(heavy, smem);
         Grid gr = plan_grid(g, heavy, NE_WARPS, smem);
         gr.blocks = (int)std::min<long long>(gr.blocks, n_big + p.n_help * p.rounds);
+        p.busy = made.add(ctl, gr);
         if (deep) k_clique_ne_heavy<true><<<gr.blocks, NE_WARPS * 32, smem, s>>>(p);
         else k_clique_ne_heavy<false><<<gr.blocks, NE_WARPS * 32, smem, s>>>(p);
         GPM_CUDA(cudaGetLastError());
-        *grid = gr;
-        launches++;
     }
     if (all > big) {
         p.first = big;
@@ -651,12 +651,10 @@ int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* 
         const long long want = (all - big + NE_LIGHT_GRAB * NE_LIGHT_WARPS - 1) / (NE_LIGHT_GRAB * NE_LIGHT_WARPS);
         Grid gr = plan_grid(g, (const void*)k_clique_ne_light, NE_LIGHT_WARPS, 0);
         gr.blocks = (int)std::min<long long>(want, gr.blocks);
+        p.busy = made.add(ctl, gr);
         k_clique_ne_light<<<gr.blocks, NE_LIGHT_WARPS * 32, 0, s>>>(p);
         GPM_CUDA(cudaGetLastError());
-        if (!launches) *grid = gr;
-        launches++;
     }
-    return launches;
 }
 
 }  // namespace gpm

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -147,7 +148,9 @@ struct alignas(128) Control {
     alignas(128) unsigned long long donations;
     unsigned long long units_done, idle_polls;
     unsigned long long word_ops;      // clique: 32-bit candidate-word AND+POPC operations
-    unsigned long long busy_ns;       // sum over warps of time spent inside work units
+    // sum over warps of time spent inside work units, per launch of the call (see Launches)
+    unsigned long long busy_ns;
+    unsigned long long busy_more[3];
     int overflow;
     int pad;
     alignas(128) unsigned long long counts[GPM_CLIQUE_MAX_K + 1];  // per clique size (clique kernel)
@@ -167,6 +170,26 @@ struct Grid {
     int blocks = 0;
     int warps_per_block = 0;
     int total_warps() const { return blocks * warps_per_block; }
+};
+
+// The launches of one call, for its statistics: each adds its warps' time to a
+// word of its own, and all of it is given on the first one's grid.
+struct Launches {
+    int n = 0;
+    Grid grid[4];
+    // the word of the next launch, of shape gr
+    unsigned long long* add(Control* ctl, const Grid& gr) {
+        grid[n] = gr;
+        return n++ == 0 ? &ctl->busy_ns : &ctl->busy_more[n - 2];
+    }
+    // Warp time on the first launch's grid: with it, 1 - busy / (warps x kernel
+    // time) is the share of all launches' warp slots that held no work.
+    uint64_t busy_ns(const Control& h) const {
+        double busy = (double)h.busy_ns;
+        for (int i = 1; i < n; i++)
+            busy += (double)h.busy_more[i - 1] * grid[0].total_warps() / std::max(1, grid[i].total_warps());
+        return (uint64_t)busy;
+    }
 };
 
 // graph.cu
@@ -216,10 +239,9 @@ void run_clique_dfs(gpm_graph* g, int k, uint64_t* count_out);   // the paper's 
 void run_clique_list(gpm_graph* g, int k_lo, int k_hi, const int32_t* d_roots, int64_t n_roots,
                      unsigned long long* d_per_root, Control* ctl, int bitmap_limit);
 // clique_nonedge.cu: whole-graph counts of sizes k_lo .. k_hi (k_hi >= 3) into
-// ctl, without the roots above the bitmap limit; returns the launches made.
-// tri (nullable, k_hi <= 5): per entry of the orientation's out-lists, += the
-// triangles on that edge.
-int launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Grid* grid, unsigned int* tri = nullptr);
+// ctl, without the roots above the bitmap limit.  tri (nullable, k_hi <= 5):
+// per entry of the orientation's out-lists, += the triangles on that edge.
+void launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Launches& made, unsigned int* tri = nullptr);
 void run_motif_monitored(gpm_graph* g, int k, double threshold, uint64_t* counts_out, MonitorStats* ms);
 
 // clique.cu / motif.cu

@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(HOM_WARPS * 32, K == 5 ? 4 : 8) k_hom(HomLaunc
     if (lane == 0) {
         atomicAdd(&p.ctl->units_done, units);
         atomicAdd(&p.ctl->word_ops, scanned);
-        atomicAdd(&p.ctl->busy_ns, gpm_globaltimer() - t0);
+        atomicAdd(p.busy, gpm_globaltimer() - t0);
     }
 }
 
@@ -532,6 +532,7 @@ void run_motif_hom(gpm_graph* g, int k, uint64_t* counts_out) {
     p.hom = r->hom;
     p.ticket = &r->ctl.next_root;
     p.ctl = &r->ctl;
+    p.busy = &r->ctl.busy_ns;
     if (k == 5) p.edges = ensure_hom_edges(g, nullptr, nullptr);
     const Grid gr = plan_hom(p, k, g->num_sms, g->cfg);
     GPM_CUDA(cudaEventRecord(g->ev0, s));

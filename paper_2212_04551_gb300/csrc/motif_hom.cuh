@@ -46,6 +46,7 @@ struct HomLaunch {
     unsigned long long* hom;              // [graph][HOM_N], zero
     unsigned long long* ticket;           // next vertex, zero
     Control* ctl;
+    unsigned long long* busy;             // this launch's warp time
 };
 
 constexpr int HOM_WARPS = 4;              // warps per block

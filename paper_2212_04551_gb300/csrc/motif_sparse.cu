@@ -35,7 +35,9 @@ constexpr long long C4_SMEM_N = 110 * 1024;   // vertices whose 16-bit counters 
 
 __global__ void k_edge_sums(const int32_t* __restrict__ off, const int32_t* __restrict__ adj,
                             const int32_t* __restrict__ outdeg, const int32_t* __restrict__ deg,
-                            const unsigned int* __restrict__ tri, int32_t n, unsigned long long* __restrict__ hom) {
+                            const unsigned int* __restrict__ tri, int32_t n, unsigned long long* __restrict__ hom,
+                            unsigned long long* __restrict__ busy) {
+    const unsigned long long t0 = gpm_globaltimer();
     __shared__ unsigned long long sum[5];
     if (threadIdx.x < 5) sum[threadIdx.x] = 0ull;
     __syncthreads();
@@ -69,6 +71,7 @@ __global__ void k_edge_sums(const int32_t* __restrict__ off, const int32_t* __re
         const int at[5] = {H_CHERRY, H_STAR3, H_PATH4, H_PAW, H_DIAMOND};
         atomicAdd(&hom[at[threadIdx.x]], sum[threadIdx.x]);
     }
+    if (threadIdx.x == 0) atomicAdd(busy, (gpm_globaltimer() - t0) * (blockDim.x / 32));
 }
 
 struct Cycle4Params {
@@ -81,6 +84,7 @@ struct Cycle4Params {
     unsigned int* counters;               // n per block (global variant), zero
     unsigned long long* ticket;
     unsigned long long* out;              // += 8 x cycles
+    unsigned long long* busy;             // this launch's warp time
 };
 
 // one scan of the paths u - v - w with v, w before u; take: c(w) is read and
@@ -122,6 +126,7 @@ __global__ void __launch_bounds__(C4_THREADS) k_cycle4(Cycle4Params p) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ int s_u[32];
     __shared__ unsigned s_mask;
+    const unsigned long long t0 = gpm_globaltimer();
     unsigned int* cnt = SMEM ? smem : p.counters + (size_t)blockIdx.x * p.n;
     if (SMEM)
         for (int i = threadIdx.x; i < (p.n + 1) / 2; i += C4_THREADS) cnt[i] = 0u;
@@ -159,7 +164,10 @@ __global__ void __launch_bounds__(C4_THREADS) k_cycle4(Cycle4Params p) {
         }
     }
     sum = gpm_warp_sum(sum);
-    if ((threadIdx.x & 31) == 0 && sum) atomicAdd(p.out, 8 * sum);
+    if ((threadIdx.x & 31) == 0) {
+        if (sum) atomicAdd(p.out, 8 * sum);
+        atomicAdd(p.busy, gpm_globaltimer() - t0);
+    }
 }
 
 // ------------------------------------------------------------------- host
@@ -206,15 +214,15 @@ void run_motif_sparse(gpm_graph* g, int k, uint64_t* counts_out) {
         tri = g->scratch_slab.as<unsigned int>();
         GPM_CUDA(cudaMemsetAsync(tri, 0, tri_bytes + cnt_bytes, s));
     }
-    Grid gr;
+    Launches made;
     GPM_CUDA(cudaEventRecord(g->ev0, s));
-    int launches = launch_clique_nonedge(g, 3, k, &r->ctl, &gr, tri);
+    launch_clique_nonedge(g, 3, k, &r->ctl, made, tri);
     const int per_sm = g->cfg.blocks_per_sm > 0 ? std::min(g->cfg.blocks_per_sm, 8) : 8;
-    k_edge_sums<<<std::max(1, std::min((g->n + 31) / 32, g->num_sms * per_sm)), 256, 0, s>>>(
+    const Grid sums{std::max(1, std::min((g->n + 31) / 32, g->num_sms * per_sm)), 8};
+    k_edge_sums<<<sums.blocks, sums.warps_per_block * 32, 0, s>>>(
         g->dag_off.as<int32_t>(), g->dag_adj.as<int32_t>(), g->dag_outdeg.as<int32_t>(), g->degree.as<int32_t>(), tri,
-        g->n, r->hom);
+        g->n, r->hom, made.add(&r->ctl, sums));
     GPM_CUDA(cudaGetLastError());
-    launches++;
     if (k == 4) {
         Cycle4Params p{};
         p.indptr = g->indptr.as<int32_t>();
@@ -226,6 +234,7 @@ void run_motif_sparse(gpm_graph* g, int k, uint64_t* counts_out) {
         p.counters = tri + tri_bytes / sizeof(unsigned int);
         p.ticket = &r->ticket;
         p.out = &r->hom[H_CYCLE4];
+        p.busy = made.add(&r->ctl, Grid{blocks, C4_THREADS / 32});
         if (smem) {
             const size_t bytes = sizeof(uint32_t) * (size_t)((g->n + 1) / 2);
             allow_shared((const void*)k_cycle4<true>, bytes);
@@ -234,7 +243,6 @@ void run_motif_sparse(gpm_graph* g, int k, uint64_t* counts_out) {
             k_cycle4<false><<<blocks, C4_THREADS, 0, s>>>(p);
         }
         GPM_CUDA(cudaGetLastError());
-        launches++;
     }
     GPM_CUDA(cudaEventRecord(g->ev1, s));
     Result h;
@@ -246,10 +254,10 @@ void run_motif_sparse(gpm_graph* g, int k, uint64_t* counts_out) {
     st.kernel_ms = ms;
     st.units_done = h.ctl.units_done;
     st.word_ops = h.ctl.word_ops;
-    st.busy_warp_ns = h.ctl.busy_ns;
-    st.kernel_launches = launches;
-    st.grid_blocks = gr.blocks;
-    st.warps_per_block = gr.warps_per_block;
+    st.busy_warp_ns = made.busy_ns(h.ctl);
+    st.kernel_launches = made.n;
+    st.grid_blocks = made.grid[0].blocks;
+    st.warps_per_block = made.grid[0].warps_per_block;
     g->stats = st;
     unsigned long long* hom = h.hom;
     const unsigned long long cherries = hom[H_CHERRY];
