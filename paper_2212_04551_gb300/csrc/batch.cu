@@ -309,17 +309,25 @@ static long long build_units(gpm_batch* b, int kc, int km, int mode, int split, 
     return (long long)codes.size();
 }
 
+// Whether this batch's motifs of size km come from the homomorphism launch
+static bool uses_hom(const gpm_batch* b, int km) {
+    return km > 0 && b->cfg.motif_agg_min > 0 && hom_applies(b->max_graph_n, b->g->max_deg, km);
+}
+
 static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     gpm_graph* g = b->g;
     const int wpb = b->cfg.warps_per_block > 0 ? b->cfg.warps_per_block : 8;
     const int bps = b->cfg.blocks_per_sm;
     const int split = std::max(1, b->cfg.batch_split);
     const int hom_k = km;
-    bool hom = km > 0 && b->cfg.motif_agg_min > 0 && hom_applies(b->max_graph_n, g->max_deg, km);
-    auto find = [&] {
-        return b->graphs.find({kc, hom_k, hom, wpb, bps, b->order_mode, b->cfg.motif_agg_min, split});
+    bool hom = uses_hom(b, km);
+    // (settings that the launches of a route do not look at are no part of the key)
+    auto key = [&] {
+        if (!hom) return std::make_tuple(kc, hom_k, false, wpb, bps, b->order_mode, b->cfg.motif_agg_min, split);
+        if (kc > hom_k) return std::make_tuple(kc, hom_k, true, wpb, bps, b->order_mode, 1, split);
+        return std::make_tuple(kc, hom_k, true, b->cfg.warps_per_block > 0 ? std::min(wpb, HOM_WARPS) : HOM_WARPS, bps, 0, 1, 1);
     };
-    auto it = find();
+    auto it = b->graphs.find(key());
     if (it != b->graphs.end()) return it->second;
 
     if (kc > 0) ensure_dag(g);
@@ -351,7 +359,7 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
         if (e.status != GPM_ENOMEM) throw;
         dev_hom.release();
         hom = false;
-        it = find();
+        it = b->graphs.find(key());
         if (it != b->graphs.end()) return it->second;
     }
     if (hom) km = 0;      // no motif units in k_batch
@@ -448,8 +456,7 @@ static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {
     cudaError_t e3 = cudaGraphInstantiate(&c.exec, graph, 0);
     cudaGraphDestroy(graph);
     check_cuda(e3, "cudaGraphInstantiate");
-    return b->graphs.emplace(std::make_tuple(kc, hom_k, hom, wpb, bps, b->order_mode, b->cfg.motif_agg_min, split),
-                             std::move(c)).first->second;
+    return b->graphs.emplace(key(), std::move(c)).first->second;
 }
 
 // One replay; results in cap.host_out.  Returns the device time (ms).
@@ -617,30 +624,37 @@ gpm_config batch_autotune(gpm_batch* b, int kc, int km, int reps, double* best_m
             best_mode = mode;
         }
     };
+    // a call served by the homomorphism launch alone has no units to order or
+    // to split, and at most HOM_WARPS warps per block
+    auto hom_alone = [&](const gpm_config& c) {
+        b->cfg = c;
+        return uses_hom(b, km) && kc <= km;
+    };
+    const bool alone = hom_alone(saved);
     // stage 1: launch shape and unit order
-    for (int mode = 0; mode < 2; mode++)
+    for (int mode = 0; mode < (alone ? 1 : 2); mode++)
         for (int wpb : {2, 4, 8, 16})
             for (int bps : {0, 1, 2}) {
+                if (alone && wpb > HOM_WARPS) continue;
                 gpm_config c = saved;
                 c.warps_per_block = wpb;
                 c.blocks_per_sm = bps;
-                // the result's split is one of stage 3's (in a call without units they all tie)
-                if (c.batch_split != 4 && c.batch_split != 16) c.batch_split = 1;
-                trial(c, mode);
+                if (alone) c.batch_split = 1;
+                trial(c, alone ? best_mode : mode);
             }
     // stage 2: class-counting threshold of the motif tail (0: leaf by leaf)
     if (km > 0) {
         const gpm_config base = best;
         const int mode = best_mode;
         for (int agg : {0, 4, 16, 64}) {
-            if (agg == base.motif_agg_min) continue;
             gpm_config c = base;
             c.motif_agg_min = agg;
+            if (agg == base.motif_agg_min || hom_alone(c)) continue;
             trial(c, mode);
         }
     }
     // stage 3: split of the heaviest roots into child ranges
-    {
+    if (!hom_alone(best)) {
         const gpm_config base = best;
         const int mode = best_mode;
         for (int split : {1, 4, 16}) {

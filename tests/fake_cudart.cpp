@@ -111,6 +111,7 @@ void fake_fail(const char* call, int at) {
 int fake_failed() { return g_failed; }
 void fake_memory_limit(size_t bytes) { g_limit = bytes; }
 size_t fake_memory_in_use() { return g_in_use; }
+int fake_calls(const char* call) { return g_calls[call]; }
 int fake_violations() { return g_violations; }
 const char* fake_log() { return g_log.c_str(); }
 void fake_clear_log() { g_log.clear(); }

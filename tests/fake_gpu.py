@@ -35,7 +35,7 @@ class FakeGpu:
             f.restype, f.argtypes = res, args
         vp, ci, sz = ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t
         for name, res, args in [("fake_reset", None, []), ("fake_fail", None, [ctypes.c_char_p, ci]),
-                                ("fake_failed", ci, []), ("fake_memory_limit", None, [sz]),
+                                ("fake_failed", ci, []), ("fake_calls", ci, [ctypes.c_char_p]), ("fake_memory_limit", None, [sz]),
                                 ("fake_memory_in_use", sz, []), ("fake_violations", ci, []),
                                 ("fake_log", ctypes.c_char_p, []), ("fake_clear_log", None, []),
                                 ("fake_on_event_record", None, [vp]), ("fake_stream", vp, [ci])]:
@@ -88,3 +88,8 @@ class FakeGpu:
     def batch_count(self, b, kc, km, graphs):
         c, m = np.zeros(graphs, np.uint64), np.zeros(graphs * 853, np.uint64)
         return self.lib.gpm_batch_count(b, kc, km, c.ctypes.data_as(gpm._u64p), m.ctypes.data_as(gpm._u64p))
+
+    def autotune(self, b, kc, km):
+        c, ms = gpm.gpm_config(), ctypes.c_double()
+        assert self.lib.gpm_batch_autotune(b, kc, km, 1, ctypes.byref(c), ctypes.byref(ms)) == gpm.GPM_OK, self.error()
+        return c

@@ -164,3 +164,31 @@ def test_launch_shapes_follow_the_configuration(gpu, n, k, kernel):
         (_, blocks, threads, _), = [x for x in gpu.log() if "k_homILi5" in x[0]]
         assert blocks <= 152 * bps and threads <= 32 * wpb
     gpu.lib.gpm_batch_destroy(b)
+
+
+def test_autotune_keeps_the_callers_split_a_candidate(gpu):
+    """Every replay takes the same time here, so that the first candidate is
+    kept: the caller's split, where roots are split at all."""
+    b = gpu.batch(*_two_paths(30))
+    gpu.configure(b, batch=True, batch_split=64)
+    assert gpu.autotune(b, 6, 4).batch_split == 64
+    gpu.lib.gpm_batch_destroy(b)
+
+
+def test_one_capture_for_settings_that_a_launch_does_not_look_at(gpu):
+    """Cliques no larger than the motifs: one homomorphism launch, whatever the
+    order, the threshold and the split."""
+    b = gpu.batch(*_two_paths(31))
+    captures = lambda: gpu.lib.fake_calls(b"cudaGraphInstantiate")
+    for cfg in (dict(), dict(batch_split=16), dict(motif_agg_min=4), dict(motif_agg_min=64, batch_split=4),
+                dict(warps_per_block=4), dict(warps_per_block=16)):
+        gpu.configure(b, batch=True, **cfg)
+        assert gpu.batch_count(b, 4, 5, 2) == gpm.GPM_OK, gpu.error()
+        assert captures() == 1
+    gpu.configure(b, batch=True, batch_split=64)
+    before = captures()
+    best = gpu.autotune(b, 4, 5)
+    # shapes of 2 and 4 warps at 0, 1 and 2 blocks per SM (one is there already), and the walk
+    assert captures() - before <= 6
+    assert best.batch_split == 1 and best.warps_per_block in (2, 4)
+    gpu.lib.gpm_batch_destroy(b)
