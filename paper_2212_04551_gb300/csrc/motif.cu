@@ -717,8 +717,8 @@ static void motif_count_noalloc(const int32_t* indptr, const int32_t* indices, i
     GPM_CUDA(cudaStreamSynchronize(s));
     if (hf[0]) fail(GPM_EINVAL, "indptr is not non-decreasing");
     if (n > 0 && ends[1] > 0) {
-        k_validate<<<std::max(1, std::min(sms * 8, (ends[1] + 255) / 256)), 256, 0, s>>>(indptr, indices, n, ends[1],
-                                                                                      flags);
+        k_validate<<<(int)std::min<int64_t>(sms * 8, ((int64_t)ends[1] + 255) / 256), 256, 0, s>>>(indptr, indices, n,
+                                                                                                   ends[1], flags);
         GPM_CUDA(cudaGetLastError());
         GPM_CUDA(cudaMemcpyAsync(hf, flags, sizeof(int), cudaMemcpyDeviceToHost, s));
         GPM_CUDA(cudaStreamSynchronize(s));

@@ -192,3 +192,12 @@ def test_one_capture_for_settings_that_a_launch_does_not_look_at(gpu):
     assert captures() - before <= 6
     assert best.batch_split == 1 and best.warps_per_block in (2, 4)
     gpu.lib.gpm_batch_destroy(b)
+
+
+def test_noalloc_checks_the_longest_list_of_entries_with_a_full_grid(gpu):
+    indptr = np.array([0, 2 ** 31 - 2], np.int32)           # (2^31 - 2) + 255 does not fit in 32 bits
+    indices, counts = np.zeros(1, np.int32), np.zeros(2, np.uint64)
+    gpu.log()
+    gpu.lib.gpm_motif_count_noalloc(indptr.ctypes.data, indices.ctypes.data, 1, 3, counts.ctypes.data_as(gpm._u64p), 2, None)
+    (_, blocks, threads, _), = [x for x in gpu.log() if "k_validate" in x[0]]
+    assert (blocks, threads) == (152 * 8, 256)
