@@ -67,11 +67,12 @@ __global__ void k_edge_sums(const int32_t* __restrict__ off, const int32_t* __re
         if ((threadIdx.x & 31) == 0 && s) atomicAdd(&sum[j], s);
     }
     __syncthreads();
-    if (threadIdx.x < 5 && sum[threadIdx.x]) {
-        const int at[5] = {H_CHERRY, H_STAR3, H_PATH4, H_PAW, H_DIAMOND};
-        atomicAdd(&hom[at[threadIdx.x]], sum[threadIdx.x]);
+    if (threadIdx.x < 6) {
+        const int at[6] = {H_CHERRY, H_STAR3, H_PATH4, H_PAW, H_DIAMOND, 0};
+        const bool time = threadIdx.x == 5;
+        const unsigned long long x = time ? (gpm_globaltimer() - t0) * (blockDim.x / 32) : sum[threadIdx.x];
+        if (x) atomicAdd(time ? busy : &hom[at[threadIdx.x]], x);
     }
-    if (threadIdx.x == 0) atomicAdd(busy, (gpm_globaltimer() - t0) * (blockDim.x / 32));
 }
 
 struct Cycle4Params {
@@ -164,10 +165,8 @@ __global__ void __launch_bounds__(C4_THREADS) k_cycle4(Cycle4Params p) {
         }
     }
     sum = gpm_warp_sum(sum);
-    if ((threadIdx.x & 31) == 0) {
-        if (sum) atomicAdd(p.out, 8 * sum);
-        atomicAdd(p.busy, gpm_globaltimer() - t0);
-    }
+    if ((threadIdx.x & 31) == 0 && sum) atomicAdd(p.out, 8 * sum);
+    if (threadIdx.x == 0) atomicAdd(p.busy, (gpm_globaltimer() - t0) * (C4_THREADS / 32));
 }
 
 // ------------------------------------------------------------------- host

@@ -20,7 +20,14 @@ def _communities(count):
     return G.disjoint_union(*[G.gnp(90, 0.6, s) for s in range(count)], *[G.gnp(30, 0.6, s) for s in range(count * 10)])
 
 
+def _one_heavy():
+    """A single root above 32 out-neighbours: the first launch has one block."""
+    return G.disjoint_union(G.complete(34), *[G.gnp(30, 0.6, s) for s in range(2500)])
+
+
 @pytest.mark.parametrize("graph,call", [
+    (_one_heavy, lambda g: gpm.gpm_clique_count(g, 4)),
+    (_one_heavy, lambda g: gpm.gpm_motif_count(g, 4)),
     (lambda: _bicliques(12, 700), lambda g: gpm.gpm_motif_count(g, 4)),         # the cycles of four take the time
     (lambda: _communities(200), lambda g: gpm.gpm_clique_count(g, 4)),
     (lambda: _communities(200), lambda g: gpm.gpm_clique_count_range(g, 3, 8))])
