@@ -40,15 +40,22 @@ static_assert(MLP_NPARAM == GPM_MLP_PARAMS, "parameter count");
 // ------------------------------------------------------------- features
 
 // triangles rooted at v in the degree orientation: sum over u in N+(v) of
-// |N+(v) & N+(u)|.  Warp per v, eight lanes per list N+(u) with 16-byte loads
-// (the lists are padded and aligned for it), every entry searched in N+(v),
-// which lies in shared memory up to TRI_LIST entries.
-constexpr int TRI_LIST = 1024;
+// |N+(v) & N+(u)|.  Warp per v.  Up to TRI_LIST entries N+(v) lies in shared
+// memory and eight lanes take a list N+(u) with 16-byte loads (the lists are
+// padded and aligned for it); above, the whole warp takes a list, whose
+// consecutive entries search nearly the same words of N+(v), in L1.
+//
+// Bound: the latency of the searches.  All root features, every list by whole
+// warps / by eight lanes, in shared memory up to 1,024 / this: R-MAT 2^16 16.4 /
+// 2.2 / 2.2 ms (the first with the core numbers of then), random graph of 30,000
+// vertices and degree 1,000 61 / 57 / 38, K_1100 14.2 / 17.4 / 13.0, random graph
+// of 8,192 vertices and degree 3,500 257 / 753 / 229.
+constexpr int TRI_LIST = 256;
 constexpr int TRI_THREADS = 256;
-__global__ void __launch_bounds__(TRI_THREADS) k_tri_root(const int32_t* __restrict__ off,
-                                                          const int32_t* __restrict__ adj,
-                                                          const int32_t* __restrict__ outdeg, int32_t n,
-                                                          float* __restrict__ tri) {
+__global__ void __launch_bounds__(TRI_THREADS, 8) k_tri_root(const int32_t* __restrict__ off,
+                                                             const int32_t* __restrict__ adj,
+                                                             const int32_t* __restrict__ outdeg, int32_t n,
+                                                             float* __restrict__ tri) {
     __shared__ int32_t s_list[TRI_THREADS / 32][TRI_LIST];
     const int lane = threadIdx.x & 31;
     int32_t* sl = s_list[threadIdx.x >> 5];
@@ -61,20 +68,29 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_root(const int32_t* __restr
             for (int t = lane; t < d; t += 32) sl[t] = adj[b + t];
         __syncwarp();
         long long c = 0;
-        for (int i = lane >> 3; i < d; i += 4) {
-            const int u = small ? sl[i] : adj[b + i];
-            const int ub = off[u], du = outdeg[u];
-            for (int t = 4 * (lane & 7); t < du; t += 32) {
-                const int4 x4 = *reinterpret_cast<const int4*>(adj + ub + t);
-                const int xs[4] = {x4.x, x4.y, x4.z, x4.w};   // padding is above every id
-#pragma unroll
-                for (int z = 0; z < 4; z++) {
-                    int lo = 0, hi = d - 1;
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if ((small ? sl[mid] : adj[b + mid]) < xs[z]) lo = mid + 1; else hi = mid;
-                    }
-                    c += (small ? sl[lo] : adj[b + lo]) == xs[z] ? 1 : 0;
+        // the entries of N+(u) for all u in N+(v), searched in `list` = N+(v)
+        auto found = [d](const auto* list, int x) {
+            int lo = 0, hi = d - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (list[mid] < x) lo = mid + 1; else hi = mid;
+            }
+            return list[lo] == x ? 1 : 0;
+        };
+        if (!small) {
+            const int32_t* list = adj + b;
+            for (int i = 0; i < d; i++) {
+                const int u = list[i];
+                const int ub = off[u], du = outdeg[u];
+                for (int t = lane; t < du; t += 32) c += found(list, adj[ub + t]);
+            }
+        } else {
+            for (int i = lane >> 3; i < d; i += 4) {
+                const int u = sl[i];
+                const int ub = off[u], du = outdeg[u];
+                for (int t = 4 * (lane & 7); t < du; t += 32) {
+                    const int4 x4 = *reinterpret_cast<const int4*>(adj + ub + t);   // padding is above every id
+                    c += found(sl, x4.x) + found(sl, x4.y) + found(sl, x4.z) + found(sl, x4.w);
                 }
             }
         }
