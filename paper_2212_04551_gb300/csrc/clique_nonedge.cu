@@ -18,7 +18,8 @@
 //     A child's members without non-edges are set aside as a number; the
 //     others are re-indexed (up to 128 of them) and counted in registers.
 //     From a set with more, members are first taken out one by one in shared
-//     memory, by the same rule, until 128 are left (ne_wide).
+//     memory, by the same rule, until 128 are left (ne_wide_step), unless three
+//     sizes are to go and nearly all would have to be (ne_wide_direct).
 //
 // The row build reads every out-list of N+(r) once: eight lanes per list with
 // 16-byte loads (the lists are padded and aligned for it), each entry tested
@@ -27,11 +28,11 @@
 // Roots above 1,024 are the list path's (clique_list.cu).
 //
 // What bounds it: the heavy launch, instruction issue and instruction fetch
-// (issue slots 0.48 busy, `no_instruction` the first stall; 2.6e10 warp
+// (issue slots 0.49 busy, `no_instruction` the first stall; 2.1e10 warp
 // instructions at k = 4..7 on the Chung-Lu graph of 10^6 vertices, where the
 // walk over the cliques took 9.5e11).  Loops whose trip count depends on data
-// are therefore not unrolled: with the compiler's unrolling the heavy kernel
-// was 401 KB of code instead of 113 KB, and 81 ms instead of 34.  The light
+// are therefore not unrolled: with the compiler's unrolling an earlier state of
+// the heavy kernel was 401 KB of code instead of 113 KB, and 81 ms instead of 46.  The light
 // launch is bound by the latency of its chain of dependent loads per root.
 // Measured, whole call on that graph: k = 4..7 1,378 -> 35 ms, k = 4 8.0 ->
 // 2.8 ms; block-model graph of 2,000 vertices, k = 6..12: 20.9 -> 0.6 ms.
@@ -55,6 +56,8 @@ constexpr int NE_WARPS = 4;           // warps per block of the heavy launch
 constexpr int NE_HELP_D = 128;        // roots above this are offered to further blocks ...
 constexpr int NE_HELP_ROUNDS = 24;    // ... this many times (k >= 6, where a child's work can be large)
 constexpr int NE_SCRATCH = 64 + 128;   // words for a second re-indexing (ne_four_again)
+constexpr int NE_DIRECT_M = 160;      // wide sets of three sizes to go: from this many members with non-edges,
+constexpr int NE_DIRECT_E = 2;        // and this many on average, the triangles are counted (ne_wide_direct)
 constexpr int NE_FILTER_WORDS = 64;   // hash filter of N+(r): 2,048 bits
 
 struct NeLaunch {
@@ -328,6 +331,45 @@ __device__ __forceinline__ NeTodo ne_node(const NeLaunch& p, NeCount& c, const N
     return m <= 32 * NE_W ? NE_INDEX : NE_WIDE;
 }
 
+// Three sizes to go, a wide set C with m members that have non-edges: where
+// these leave little to a closed form -- taken out one by one, nearly all would
+// have to go -- the triangles of the graph among C are counted directly, as the
+// walk counts them.  Returns their number, the edges and the members (28, 20
+// and 12 bits from the lowest), 0 if the set is better taken apart.  CU: w words
+// of scratch.  Out of line: the code of the other sets is bound by its fetch.
+//
+// 5-cliques, walk / taken apart / this where it applies: complete multipartite graphs,
+// 600 vertices in parts of 100 47 / 91 / 33 ms, in parts of 5 103 / 217 / 80, in
+// parts of 2 66 / 2.4 / 2.7; G(600, 0.8) 41 / 67 / 26, G(900, 0.7) 93 / 126 / 43.
+// From 129, 160 or 200 members: parts of 50, 300 vertices, k = 5 3.8 / 3.7 / 5.0,
+// k = 6 11.0 / 8.8 / 8.8.
+__device__ __noinline__ unsigned long long ne_wide_direct(const uint32_t* rows, int ws, int w, const uint32_t* C,
+                                                          uint32_t* CU, uint16_t* mem, int m, int lane) {
+    const int n = ne_members(C, w, mem, lane);
+    unsigned e2 = 0;
+    for (int t = lane; t < n; t += 32) e2 += (unsigned)ne_degree(rows, ws, w, C, mem[t]);
+    e2 = __reduce_add_sync(GPM_FULL_MASK, e2);
+    if (e2 < (unsigned)(NE_DIRECT_E * m)) return 0;
+    unsigned t = 0;
+    for (int i = 0; i < n - 2; i++) {
+        const int u = mem[i];
+        const uint32_t* ru = rows + u * ws;
+        if (lane < w) CU[lane] = C[lane] & ru[lane];
+        __syncwarp();
+        for (int j = i + 1 + lane; j < n; j += 32) {
+            const int v = mem[j];
+            if (!((CU[v >> 5] >> (v & 31)) & 1u)) continue;
+            const uint32_t* rv = rows + v * ws;
+            t += __popc(CU[v >> 5] & rv[v >> 5] & (0xfffffffeu << (v & 31)));
+#pragma unroll 4
+            for (int z = (v >> 5) + 1; z < w; z++) t += __popc(CU[z] & rv[z]);
+        }
+        __syncwarp();
+    }
+    t = __reduce_add_sync(GPM_FULL_MASK, t);
+    return (unsigned long long)t | (unsigned long long)((unsigned)n * (n - 1) - e2) / 2 << 28 | (unsigned long long)n << 48;
+}
+
 // One step on the wide set C of traversal size lv (its members in k.wide,
 // `left` of n not taken out yet): NE_DONE if it is finished, NE_INDEX if at
 // most 128 members with non-edges are left (now in k.mem), else NE_WIDE: the
@@ -389,6 +431,15 @@ __device__ __forceinline__ void ne_child(const NeLaunch& p, NeCount& c, const Ne
 #pragma unroll 1
     for (;;) {
         NeTodo todo = ne_node(p, c, k, rows, w, k.cand + h * w, h, m, a, lane);
+        if (todo == NE_WIDE && h + 3 == p.ne.k_hi && m >= NE_DIRECT_M) {
+            const unsigned long long r = ne_wide_direct(rows, p.ws, w, k.cand + h * w, k.cand + (h + 1) * w, k.mem, m, lane);
+            if (r) {
+                const int j = lane - h;                // cliques of h + j members
+                c.size = gpm_add_cc(c.size, j == 3 ? r & 0xfffffffu : j == 2 ? (r >> 28) & 0xfffffu : j == 1 ? r >> 48
+                                            : j == 0 ? 1ull : 0ull, c.ovf);
+                todo = NE_DONE;
+            }
+        }
         bool load = todo == NE_WIDE, over = false;
         if (load) lv = h;
 #pragma unroll 1
