@@ -309,9 +309,22 @@ static long long build_units(gpm_batch* b, int kc, int km, int mode, int split, 
     return (long long)codes.size();
 }
 
-// Whether this batch's motifs of size km come from the homomorphism launch
+// Whether this batch's motifs of size km come from the homomorphism launch.
+// Its arrays have an entry per vertex of the largest graph, so large graphs
+// leave few warps resident, and the walk keeps up where it has little to do:
+// sets of 4 and 5 on graphs little denser than paths, or sets of 3, which cost
+// it one scan of half the lists.  Walk / homomorphism launch, 64,000 vertices in
+// graphs of n at average degree d, us: k = 3, n = 2,000 d = 80 660 / 570, n =
+// 4,000 d = 40 390 / 370, d = 80 680 / 980, n = 16,384 d = 16 550 / 350, d = 40
+// 740 / 920; k = 4, n = 2,000 d = 2 230 / 150, n = 4,000 d = 2 220 / 260, d = 4
+// 460 / 310, n = 16,384 d = 4 680 / 800, d = 8 1,880 / 1,000; k = 5, n = 2,000
+// d = 2 230 / 180, n = 4,000 d = 2 250 / 360, d = 4 2,740 / 650.
 static bool uses_hom(const gpm_batch* b, int km) {
-    return km > 0 && b->cfg.motif_agg_min > 0 && hom_applies(b->max_graph_n, b->g->max_deg, km);
+    const int n = b->max_graph_n;
+    if (km <= 0 || b->cfg.motif_agg_min <= 0 || !hom_applies(n, b->g->max_deg, km)) return false;
+    const double avg = (double)b->g->nnz / std::max(b->g->n, 1);
+    if (km == 3) return n <= 2048 || avg <= 32.0;
+    return n <= 3000 || avg >= (km == 4 && n > 12288 ? 6.0 : 3.0);
 }
 
 static gpm_batch::Captured& capture(gpm_batch* b, int kc, int km) {

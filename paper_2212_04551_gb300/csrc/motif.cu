@@ -317,7 +317,8 @@ __global__ void k_motif_seed(const int32_t* __restrict__ roots, long long n_coun
 static bool motif_from_sums(gpm_graph* g, int k, uint64_t* counts_out) {
     const bool had_dag = g->dag_ready;
     try {
-        if (hom_applies(g->n, g->max_deg, k) && (k == 5 || g->max_deg <= (k == 3 ? HOM_HUB_D3 : HOM_HUB_D4))) {
+        if (hom_applies(g->n, g->max_deg, k) && (k == 5 || (g->max_deg <= (k == 3 ? HOM_HUB_D3 : HOM_HUB_D4) &&
+                                                             g->n <= (k == 3 ? HOM_SUMS_N3 : HOM_SUMS_N4)))) {
             run_motif_hom(g, k, counts_out);
             return true;
         }

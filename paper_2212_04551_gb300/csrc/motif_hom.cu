@@ -27,9 +27,12 @@
 // 2^14 vertices and degrees up to 2^10, which bounds every homomorphism count
 // (n d^(k-1)) by 2^54, so that 64-bit sums are exact.
 //
-// What bounds it: the latency of the loads and lookups (one warp per vertex, 16
-// warps per SM at 128 registers for k = 5; issue slots 0.3 busy), hence several
-// entries per lane in flight in every scan.
+// What bounds it: the latency of the loads and lookups (one warp per vertex;
+// issue slots 0.3 busy), hence several entries per lane in flight in every scan.
+// The warps in flight are limited by their arrays in shared memory, 8 bytes per
+// vertex of the graph and the rows: 8 warps per SM on the block-model graph of
+// 2,000 vertices (21.7 KB each), 1 at 2^14; on small graphs by the 128
+// registers of k = 5 (16).
 // Measured, whole call, the walk / this: G(516, 1200) k = 4 857 / 33 us;
 // block-model graph of 2,000 vertices k = 5 199 / 1.4 ms; 4,096 small graphs,
 // 4-cliques and 5-motifs 150 / 6.6 ms.
@@ -341,9 +344,9 @@ __device__ __forceinline__ void hom_vertex(const HomLaunch& p, const HomWarp& k,
                     int done = 0;
                     for (; q < e; q += 8) {
                         const int x = p.indices[q] - base;
-                        if (x >= hi) break;
-                        // (an unchecked graph's lists may not be sorted)
-                        if (x >= lo) atomicOr(&k.M[(x - lo) * w + (i >> 5)], 1u << (i & 31));
+                        // (x < lo: only in an unchecked graph, whose lists may not be sorted)
+                        if ((unsigned)(x - lo) >= (unsigned)(hi - lo)) break;
+                        atomicOr(&k.M[(x - lo) * w + (i >> 5)], 1u << (i & 31));
                         done++;
                     }
                     if (i < d && done) atomicAdd(&k.at[i], done);
@@ -383,11 +386,11 @@ __global__ void __launch_bounds__(HOM_WARPS * 32, K == 5 ? 4 : 8) k_hom(HomLaunc
     k.seen = k.idx + n4;
     k.c = mine + n4;
     k.t = reinterpret_cast<int*>(k.c + n4);
-    k.at = k.t + d4;
+    k.at = K == 3 ? reinterpret_cast<int*>(mine + n4 / 2) : k.t + d4;     // (k = 3: idx, at and end only)
     k.end = k.at + d4;
     k.L = reinterpret_cast<uint32_t*>(k.end + d4);
     k.M = k.L + p.maxd * (w | 1);
-    for (int i = lane; i < (K == 3 ? n4 : 2 * n4); i += 32) mine[i] = 0u;
+    for (int i = lane; i < (K == 3 ? n4 / 2 : 2 * n4); i += 32) mine[i] = 0u;
     __syncwarp();
     HomSums a;
 #pragma unroll
@@ -464,7 +467,7 @@ int hom_m_words(int n, int d) {
 
 int hom_warp_words(int n, int d, int k) {
     const int n4 = (n + 3) & ~3, d4 = (d + 3) & ~3, w = (d + 31) >> 5;
-    if (k == 3) return n4 + n4 + 3 * d4;                 // (no rows)
+    if (k == 3) return n4 / 2 + 2 * d4;                  // (idx, at and end only)
     return 2 * n4 + 3 * d4 + ((d * (w | 1) + (k == 5 ? hom_m_words(n, d) : 0) + 3) & ~3);
 }
 

@@ -57,6 +57,13 @@ constexpr int HOM_MAX_D = 1024;           // largest degree (bit rows over a nei
 // 74 / 78 us, 123 110 / 93, 931 6,400 / 230; block-model graph, degree 100: 200 /
 // 250; k = 3: degree 123 53 / 77, 216 82 / 80, 931 450 / 155.
 constexpr int HOM_HUB_D3 = 210, HOM_HUB_D4 = 110;
+// And with more vertices than this, whose arrays leave few warps resident.
+// Random graphs of average degree 6 / 16 / 60, these and edge sums in us: k = 3,
+// n = 4,000: 58, 65 / 60, 74 / 85, 152; 8,000: 60, 73 / 64, 71 / 136, 160; 12,000:
+// 74, 67 / 86, 72 / 238, 188; 16,384: 116, 71 / 146, 75 / 534, 216; k = 4, n = 4,000:
+// 64, 120 / 84, 136 / 384, 265; 6,000: 71, 142 / 111, 179 / 521, 383; 8,000: 127, 174 /
+// 200, 191 / 1,218, 413; 16,384: 371, 206 / 632, 244 / 4,525, 686.
+constexpr int HOM_SUMS_N3 = 8192, HOM_SUMS_N4 = 6144;
 
 // Whether graphs of at most n vertices and degree d are counted this way.
 bool hom_applies(long long n, long long d, int k);

@@ -201,3 +201,35 @@ def test_noalloc_checks_the_longest_list_of_entries_with_a_full_grid(gpu):
     gpu.lib.gpm_motif_count_noalloc(indptr.ctypes.data, indices.ctypes.data, 1, 3, counts.ctypes.data_as(gpm._u64p), 2, None)
     (_, blocks, threads, _), = [x for x in gpu.log() if "k_validate" in x[0]]
     assert (blocks, threads) == (152 * 8, 256)
+
+
+def _ring_of_cliques(n, degree):
+    """n vertices of the given even degree (a circulant)."""
+    steps = np.arange(1, degree // 2 + 1)
+    v = np.arange(n)[:, None]
+    return np.arange(n + 1) * degree, np.sort(np.c_[(v + steps) % n, (v - steps) % n], axis=1).ravel()
+
+
+@pytest.mark.parametrize("n,degree,k,hom", [
+    (2048, 64, 3, True), (2100, 64, 3, False), (2100, 32, 3, True), (16384, 32, 3, True), (16384, 34, 3, False),
+    (3000, 2, 4, True), (3002, 2, 4, False), (3002, 4, 4, True), (12290, 4, 4, False), (12290, 6, 4, True),
+    (3000, 2, 5, True), (3002, 2, 5, False), (16384, 4, 5, True), (300, 4, 6, False)])
+def test_route_of_a_batchs_motifs(gpu, n, degree, k, hom):
+    """Size and average degree choose between the homomorphism launch and the walk."""
+    ip, ix = _ring_of_cliques(n, degree)
+    b = gpu.batch([0, n], ip, ix)
+    gpu.log()
+    assert gpu.batch_count(b, 0, k, 1) == gpm.GPM_OK, gpu.error()
+    names = [x[0] for x in gpu.log()]
+    assert any("5k_hom" in x for x in names) == hom and any("7k_batch" in x for x in names) != hom
+    gpu.lib.gpm_batch_destroy(b)
+
+
+@pytest.mark.parametrize("n,k,hom", [(8192, 3, True), (8194, 3, False), (6144, 4, True), (6146, 4, False), (16384, 5, True)])
+def test_route_of_a_graphs_motifs(gpu, n, k, hom):
+    g = gpu.graph(*_ring_of_cliques(n, 4))
+    gpu.log()
+    assert gpu.motifs(g, k) == gpm.GPM_OK, gpu.error()
+    names = [x[0] for x in gpu.log()]
+    assert any("5k_hom" in x for x in names) == hom and any("11k_edge_sums" in x for x in names) != hom
+    gpu.lib.gpm_graph_destroy(g)
