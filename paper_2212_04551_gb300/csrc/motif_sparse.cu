@@ -127,7 +127,8 @@ __global__ void __launch_bounds__(C4_THREADS) k_cycle4(Cycle4Params p) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ int s_u[32];
     __shared__ unsigned s_mask;
-    const unsigned long long t0 = gpm_globaltimer();
+    // (end minus start, added up modulo 2^64: nothing is held over the loops)
+    if (threadIdx.x == 0) atomicAdd(p.busy, 0ull - gpm_globaltimer() * (C4_THREADS / 32));
     unsigned int* cnt = SMEM ? smem : p.counters + (size_t)blockIdx.x * p.n;
     if (SMEM)
         for (int i = threadIdx.x; i < (p.n + 1) / 2; i += C4_THREADS) cnt[i] = 0u;
@@ -166,7 +167,7 @@ __global__ void __launch_bounds__(C4_THREADS) k_cycle4(Cycle4Params p) {
     }
     sum = gpm_warp_sum(sum);
     if ((threadIdx.x & 31) == 0 && sum) atomicAdd(p.out, 8 * sum);
-    if (threadIdx.x == 0) atomicAdd(p.busy, (gpm_globaltimer() - t0) * (C4_THREADS / 32));
+    if (threadIdx.x == 0) atomicAdd(p.busy, gpm_globaltimer() * (C4_THREADS / 32));
 }
 
 // ------------------------------------------------------------------- host
