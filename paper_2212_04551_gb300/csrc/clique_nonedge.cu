@@ -422,7 +422,10 @@ __device__ __forceinline__ NeTodo ne_wide_step(const NeLaunch& p, NeCount& c, co
 }
 
 // All cliques of the set in cand[2] (traversals of size 2), depth first over
-// wide sets.
+// wide sets.  DIRECT: with the call of ne_wide_direct, around which the loops
+// keep fewer values in registers (Chung-Lu, 10^6 vertices, k = 5 without / with:
+// 5.91 / 6.07 ms, k = 4..7 33.9 / 33.4).
+template <bool DIRECT>
 __device__ __forceinline__ void ne_child(const NeLaunch& p, NeCount& c, const NeWarp& k, const uint32_t* rows, int w,
                                          int lane) {
     int h = 2;                 // the size of the set looked at
@@ -431,7 +434,7 @@ __device__ __forceinline__ void ne_child(const NeLaunch& p, NeCount& c, const Ne
 #pragma unroll 1
     for (;;) {
         NeTodo todo = ne_node(p, c, k, rows, w, k.cand + h * w, h, m, a, lane);
-        if (todo == NE_WIDE && h + 3 == p.ne.k_hi && m >= NE_DIRECT_M) {
+        if (DIRECT && todo == NE_WIDE && h + 3 == p.ne.k_hi && m >= NE_DIRECT_M) {
             const unsigned long long r = ne_wide_direct(rows, p.ws, w, k.cand + h * w, k.cand + (h + 1) * w, k.mem, m, lane);
             if (r) {
                 const int j = lane - h;                // cliques of h + j members
@@ -473,7 +476,7 @@ __device__ __forceinline__ void ne_child(const NeLaunch& p, NeCount& c, const Ne
 // DEEP: three sizes or more to go below a child (k >= 5); without, neither the
 // re-indexed rows nor their registers are there (48 instead of 96), and twice
 // the warps are resident: k = 4 on the Chung-Lu graph 4.0 -> 2.8 ms.
-template <bool DEEP>
+template <bool DEEP, bool DIRECT>
 __global__ void __launch_bounds__(NE_WARPS * 32, DEEP ? 5 : 10) k_clique_ne_heavy(NeLaunch p) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ unsigned long long s_pos;
@@ -607,7 +610,7 @@ __global__ void __launch_bounds__(NE_WARPS * 32, DEEP ? 5 : 10) k_clique_ne_heav
                 }
                 __syncwarp();
                 if (DEEP) {
-                    ne_child(p, c, k, rows, w, lane);
+                    ne_child<DIRECT>(p, c, k, rows, w, lane);
                 } else {
                     int m, a;
                     ne_node(p, c, k, rows, w, C, 2, m, a, lane);   // two sizes to go at most: counted
@@ -679,7 +682,14 @@ void launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Launc
         p.w = (p.maxd + 31) / 32;
         p.ws = p.w | 1;
         const bool deep = k_hi >= 5;
-        const void* heavy = deep ? (const void*)k_clique_ne_heavy<true> : (const void*)k_clique_ne_heavy<false>;
+        // A child's set has fewer members than its root's list: lists well above
+        // NE_DIRECT_M, or an eighth of them above it (complete multipartite graphs and
+        // G(n, 0.5 .. 0.95) of 250 to 1,200 vertices: 0.37 to 0.78; the core of the
+        // Chung-Lu graph of 10^6: 0.08, lists of up to 297).
+        const bool direct = deep && (g->max_outdeg > 2 * NE_DIRECT_M ||
+                                     8 * (roots_at_least(g, NE_DIRECT_M + 1) - above) >= n_big);
+        const void* heavy = !deep ? (const void*)k_clique_ne_heavy<false, false>
+                            : direct ? (const void*)k_clique_ne_heavy<true, true> : (const void*)k_clique_ne_heavy<true, false>;
         p.warp_words = ne_warp_words(p.maxd, p.w, deep);
         p.n_help = std::max(0ll, roots_at_least(g, NE_HELP_D + 1) - above);
         p.rounds = k_hi >= 6 ? NE_HELP_ROUNDS : 0;
@@ -691,8 +701,9 @@ void launch_clique_nonedge(gpm_graph* g, int k_lo, int k_hi, Control* ctl, Launc
         Grid gr = plan_grid(g, heavy, NE_WARPS, smem);
         gr.blocks = (int)std::min<long long>(gr.blocks, n_big + p.n_help * p.rounds);
         p.busy = made.add(ctl, gr);
-        if (deep) k_clique_ne_heavy<true><<<gr.blocks, NE_WARPS * 32, smem, s>>>(p);
-        else k_clique_ne_heavy<false><<<gr.blocks, NE_WARPS * 32, smem, s>>>(p);
+        if (!deep) k_clique_ne_heavy<false, false><<<gr.blocks, NE_WARPS * 32, smem, s>>>(p);
+        else if (direct) k_clique_ne_heavy<true, true><<<gr.blocks, NE_WARPS * 32, smem, s>>>(p);
+        else k_clique_ne_heavy<true, false><<<gr.blocks, NE_WARPS * 32, smem, s>>>(p);
         GPM_CUDA(cudaGetLastError());
     }
     if (all > big) {

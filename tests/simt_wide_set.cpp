@@ -53,7 +53,7 @@ int main(int argc, char** argv) {
         __syncwarp();
         NeCount c;
         c.acc[0] = before;
-        ne_child(p, c, k, rows.data(), p.w, lane);
+        ne_child<true>(p, c, k, rows.data(), p.w, lane);
         most = max(most, c.acc[0] < 0 ? -c.acc[0] : c.acc[0]);
         ne_fold(p.ne, c, lane);
         if (lane == 6) counted = c.size;
