@@ -96,8 +96,9 @@ gpm_status gpm_graph_info(const gpm_graph* g, int32_t* n, int64_t* m, int32_t* m
  * their out-neighbourhood in shared memory, branching on the non-edges of the
  * candidate sets (with a clique_tail, clique_compact, clique_compact3 or
  * clique_cpl other than the default, which choose among the tails of the walk,
- * or another root order: by walking the cliques instead); roots above that, in the same call, by sorted-list intersection (the paper's
- * extension arrays) with per-warp lists in device memory.  out_count: host pointer to one uint64.
+ * or another root order: by walking the cliques instead); roots above that, in
+ * the same call, by sorted-list intersection (the paper's extension arrays) with
+ * per-warp lists in device memory.  out_count: host pointer to one uint64.
  * Errors: GPM_EINVAL, GPM_ENOMEM, GPM_ECUDA, GPM_ETIMEOUT, GPM_EOVERFLOW.
  */
 gpm_status gpm_clique_count(gpm_graph* g, int k, uint64_t* out_count);
